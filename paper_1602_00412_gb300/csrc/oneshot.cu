@@ -244,7 +244,7 @@ int sfd_orthonormalize(int64_t rows, int32_t k, float* X, int32_t ld) {
     // next two make it orthonormal to fp32 accuracy
     for (int pass = 0; pass < 3; ++pass) {
       gram(X, ld, map, rows, ws.small_a, ws, s);
-      chol_inv(ws.small_a, k, ws.small_b, ws.eig_work, ws.flags, s, true);  // FP64 factor
+      chol_inv(ws.small_a, k, ws.small_b, ws.eig_work, ws.flags, s, true);
       gemm_ts(X, ld, map, rows, ws.small_b, k, tmp, ld, s);
       SFD_CUDA(cudaMemcpy2DAsync(X, ld * sizeof(float), tmp, ld * sizeof(float), k * sizeof(float),
                                  rows, cudaMemcpyDeviceToDevice, s));

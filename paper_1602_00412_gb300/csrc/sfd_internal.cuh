@@ -209,15 +209,13 @@ void gemm_ts_tc(const float* X, int ldx, ColMap map, int64_t rows, const float* 
                 bool split = false, bool accumulate = false);
 // Cholesky of G + shift (k x k) and the inverse of the factor: Rinv (k x k
 // row-major, upper triangular) with G + shift = R^T R. flags[1] counts pivots
-// clamped. fp64: factorisation and inverse in double (one CTA; work holds
-// k (k|1) doubles when they do not fit in shared memory), else fp32.
+// clamped. accurate (k <= 256): factor and inverse in two-float arithmetic (48
+// significant bits), else fp32. work: k (k | 1) floats.
 void chol_inv(const float* G, int k, float* Rinv, float* work, int* flags, cudaStream_t s,
-              bool fp64 = false);
-// The blocked one-CTA form used by chol_inv for k <= 128.
-void chol_inv_blk(const float* G, int k, float* Rinv, int* flags, cudaStream_t s,
-                  bool fp64 = false);
-// Whether the blocked form fits one CTA's shared memory (fp64: k <= 112).
-bool chol_blk_supported(int k, bool fp64);
+              bool accurate = false);
+// The blocked one-CTA form of chol_inv (k <= 256).
+void chol_inv_blk(const float* G, int k, float* Rinv, float* work, int* flags, cudaStream_t s,
+                  bool accurate = false);
 // Largest nwant eigenpairs of the symmetric n x n S: evals (descending),
 // evecs n x nwant row-major. psd: S is a Gram matrix (positive semi-definite),
 // which allows the one-sided Jacobi path for n <= 128; otherwise (or for
