@@ -27,9 +27,9 @@ namespace {
 constexpr int kNoAllocMaxN = 256;
 
 // An upper bound of symeig_work_floats(256, 256), the eigensolver's scratch
-// for n = nwant = 256 (reflectors, eigenvector blocks, Gram and factor, an
-// n x (n|1) matrix when it does not fit in shared memory), ~2.1 MB; every
-// call checks the bound.
+// for n = nwant = 256 (reflectors and their joining factors, three eigenvector
+// blocks, Gram and factor, the factor's n x (n|1) scratch), ~2.1 MB; every call
+// checks the bound.
 constexpr size_t kNoAllocFloats = (size_t)kNoAllocMaxN * kNoAllocMaxN + kNoAllocMaxN +
                                   6 * (size_t)kNoAllocMaxN * kNoAllocMaxN +
                                   (size_t)kNoAllocMaxN * (kNoAllocMaxN | 1);

@@ -218,7 +218,7 @@ void chol_inv_blk(const float* G, int k, float* Rinv, float* work, int* flags, c
                   bool accurate = false);
 // Largest nwant eigenpairs of the symmetric n x n S: evals (descending),
 // evecs n x nwant row-major. psd: S is a Gram matrix (positive semi-definite),
-// which allows the one-sided Jacobi path for n <= 128; otherwise (or for
+// which allows the one-sided Jacobi path for n <= 64; otherwise (or for
 // larger n) tridiagonalisation + bisection + inverse iteration.
 void symeig(const float* S, int n, int nwant, float* evals, float* evecs, float* work,
             cudaStream_t s, bool psd = false);
