@@ -71,70 +71,198 @@ __global__ void k_gauss_fill(float* __restrict__ out, int64_t rows, int cols, in
 }
 
 // ------------------------------------------------------------------ Gram
-// 128 x 128 output tiles, 16 x 16 threads with 8 x 8 register micro-tiles:
-// per staged row each thread does 64 FMAs for 4 float4 shared loads.
-constexpr int kT = 128;  // output tile
-constexpr int kR = 16;   // rows (Gram) / inner dimension (GEMM) per stage
-constexpr int kGramBlocks = 304;  // split-K blocks per Gram, ~2 per SM
+// 8 x 8 register tiles of the upper triangle of G, one per thread: 7 (7 + 1) / 2 = 28
+// of them for n = 50, 325 for n = 200, where 128 x 128 tiles computed 2.4 times as many
+// products. Rows arrive 16 at a time through a ring of cp.async
+// stages. A row of a stage holds the first four columns of every group of eight, then
+// the second four, so that neighbouring tiles' float4 loads use different banks. The
+// multiply-adds are packed two columns at a time (half the issue slots; each is rounded
+// as fmaf) and bound the kernel: 64 per thread and row against 4 shared float4 loads.
+// Cold, with its reduction: 100,000 x 200 127 us (31 TFLOP/s over both triangles; 438 in
+// 128 x 128 tiles), 20,000 x 100 27 us (49), 2,000 x 50 12 us.
+constexpr int kT = 128;  // output tile of the tensor-core Grams' partials
+constexpr int kG8 = 8;
+constexpr int kGRows = 16;    // rows per stage
+constexpr int kGStages = 3;
+constexpr int kGramBlocks = 304;  // CTAs of a Gram, about 2 per SM
 
-__device__ __forceinline__ void fma8x8(float (&acc)[8][8], const float4& a0, const float4& a1,
-                                       const float4& b0, const float4& b1) {
-  const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-  const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+// acc[0..1] += a (b0, b1)
+__device__ __forceinline__ void pair_fma(float2& acc, float a, float b0, float b1) {
+  asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
+      "mov.b64 ra, {%2, %2};\n\tmov.b64 rb, {%3, %4};\n\tmov.b64 rc, {%0, %1};\n\t"
+      "fma.rn.f32x2 rc, ra, rb, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+      : "+f"(acc.x), "+f"(acc.y)
+      : "f"(a), "f"(b0), "f"(b1));
+}
+
+__device__ __forceinline__ void async_copy4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(in ? 4 : 0));
+}
+__device__ __forceinline__ void async_copy8(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(bytes));
+}
+__device__ __forceinline__ void async_copy16(float* dst, const float* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(bytes));
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::); }
+template <int N>
+__device__ __forceinline__ void async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Columns 4 c4 .. 4 c4 + 3 of row g of the operand (zero past n columns or when !in) to
+// dst, in copies of vec columns: 4 (or 2) when rows of both blocks start on 16- (8-)
+// byte boundaries and the first block's width is a multiple of that, or it is the
+// only one; else 1.
+__device__ __forceinline__ void async_cols(float* dst, const float* X, int ldx, const ColMap& map,
+                                           int64_t g, int c4, bool in, int vec) {
+  const int n = map.total(), c = 4 * c4;
+  auto src_of = [&](int cc) {
+    return cc < map.k0 ? X + g * ldx + cc : map.x1 + g * map.ld1 + (cc - map.k0);
+  };
+  auto left = [&](int cc) { return in && cc < n ? (cc < map.k0 ? map.k0 : n) - cc : 0; };
+  if (vec == 4) {
+    const int w = min(4, left(c));
+    async_copy16(dst, w > 0 ? src_of(c) : X, 4 * w);
+  } else if (vec == 2) {
+#pragma unroll
+    for (int t = 0; t < 4; t += 2) {
+      const int w = min(2, left(c + t));
+      async_copy8(dst + t, w > 0 ? src_of(c + t) : X, 4 * w);
+    }
+  } else {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const bool ok = left(c + t) > 0;
+      async_copy4(dst + t, ok ? src_of(c + t) : X, ok);
+    }
+  }
+}
+
+// partial[chunk][tile][64]: tiles of the upper triangle in row-major order.
+__global__ void __launch_bounds__(512)
+    k_gram_tri(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
+               int64_t rows_per_chunk, int ntiles, int vec, float* __restrict__ partial) {
+  extern __shared__ __align__(16) float sm[];
+  const int n = map.total(), ng = (n + kG8 - 1) / kG8;
+  const int rs = ng * kG8, ps = ng * 4;  // floats per row and per half of it
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int slot = (int)(blockIdx.y * blockDim.x) + tid, e = min(slot, ntiles - 1);
+  int ti = 0, start = 0;
+  {  // row ti of the triangle starts at ti ng - ti (ti - 1) / 2
+    const float h = (float)ng + 0.5f;
+    ti = max(0, (int)(h - sqrtf(fmaxf(h * h - 2.f * (float)e, 0.f))) - 1);
+    start = ti * ng - ti * (ti - 1) / 2;
+    while (start + (ng - ti) <= e) { start += ng - ti; ++ti; }
+  }
+  const int tj = ti + (e - start);
+  const int64_t r_beg = (int64_t)blockIdx.x * rows_per_chunk;
+  const int64_t r_end = min(rows, r_beg + rows_per_chunk);
+  const int nst = (int)((r_end - r_beg + kGRows - 1) / kGRows);
+  auto load = [&](int st) {
+    float* buf = sm + (st % kGStages) * kGRows * rs;
+    for (int r = warp; r < kGRows; r += nw) {
+      const int64_t g = r_beg + (int64_t)st * kGRows + r;
+      for (int c4 = lane; c4 < 2 * ng; c4 += 32)
+        async_cols(buf + r * rs + (c4 & 1) * ps + (c4 >> 1) * 4, X, ldx, map, g, c4, g < r_end, vec);
+    }
+  };
+  float2 acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-}
-
-__global__ void __launch_bounds__(256, 2)
-    k_gram_tiles(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
-                 int64_t rows_per_chunk, int ntiles, int npairs, float* __restrict__ partial) {
-  __shared__ __align__(16) float As[kR][kT];
-  __shared__ __align__(16) float Bs[kR][kT];
-  const int tp = blockIdx.y, chunk = blockIdx.x;
-  // (ti, tj), ti <= tj, from the row-major index over the upper triangle of tiles
-  int ti = 0, start = 0;
-  while (start + (ntiles - ti) <= tp) { start += ntiles - ti; ++ti; }
-  const int tj = ti + (tp - start);
-  const bool diag = ti == tj;
-  const int n = map.total();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float acc[8][8] = {};
-  const int64_t r_beg = (int64_t)chunk * rows_per_chunk;
-  const int64_t r_end = min(rows, r_beg + rows_per_chunk);
-  float (*Bp)[kT] = diag ? As : Bs;
-  for (int64_t r0 = r_beg; r0 < r_end; r0 += kR) {
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int q = 0; q < (kR * kT) / 256; ++q) {
-      const int li = threadIdx.x + q * 256;
-      const int rr = li / kT, cc = li % kT;
-      const int64_t g = r0 + rr;
-      const int ca = ti * kT + cc;
-      As[rr][cc] = (g < r_end && ca < n) ? map.at(X, ldx, g, ca) : 0.f;
-      if (!diag) {
-        const int cb = tj * kT + cc;
-        Bs[rr][cc] = (g < r_end && cb < n) ? map.at(X, ldx, g, cb) : 0.f;
+  for (int st = 0; st < kGStages - 1; ++st) {
+    if (st < nst) load(st);
+    async_commit();
+  }
+  for (int st = 0; st < nst; ++st) {
+    async_wait<kGStages - 2>();
+    __syncthreads();  // stage st has landed, and everyone is done with stage st - 1
+    if (st + kGStages - 1 < nst) load(st + kGStages - 1);
+    async_commit();
+    const float* buf = sm + (st % kGStages) * kGRows * rs;
+    // the next row's operands are on their way while this row's products are formed
+    float4 f[2][4];
+    auto fetch = [&](int r, float4 (&q)[4]) {
+      const float* row = buf + r * rs;
+      q[0] = *reinterpret_cast<const float4*>(row + ti * 4);
+      q[1] = *reinterpret_cast<const float4*>(row + ps + ti * 4);
+      q[2] = *reinterpret_cast<const float4*>(row + tj * 4);
+      q[3] = *reinterpret_cast<const float4*>(row + ps + tj * 4);
+    };
+    fetch(0, f[0]);
+#pragma unroll 2
+    for (int i = 0; i < kGRows; ++i) {
+      const float4(&q)[4] = f[i & 1];
+      fetch(min(i + 1, kGRows - 1), f[(i + 1) & 1]);
+      const float a[8] = {q[0].x, q[0].y, q[0].z, q[0].w, q[1].x, q[1].y, q[1].z, q[1].w};
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        pair_fma(acc[c][0], a[c], q[2].x, q[2].y);
+        pair_fma(acc[c][1], a[c], q[2].z, q[2].w);
+        pair_fma(acc[c][2], a[c], q[3].x, q[3].y);
+        pair_fma(acc[c][3], a[c], q[3].z, q[3].w);
       }
     }
-    __syncthreads();
-#pragma unroll 4
-    for (int rr = 0; rr < kR; ++rr) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[rr][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[rr][ty * 8 + 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bp[rr][tx * 8]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bp[rr][tx * 8 + 4]);
-      fma8x8(acc, a0, a1, b0, b1);
-    }
-    __syncthreads();
   }
-  float* out = partial + ((int64_t)chunk * npairs + tp) * (kT * kT);
+  async_wait<0>();
+  if (slot >= ntiles) return;
+  float4* out = reinterpret_cast<float4*>(partial + ((int64_t)blockIdx.x * ntiles + e) * 64);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    float4* o = reinterpret_cast<float4*>(&out[(ty * 8 + i) * kT + tx * 8]);
-    o[0] = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    o[1] = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+    out[2 * i] = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+    out[2 * i + 1] = make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y);
   }
+}
+
+// G = sum over chunks of a tile's partials, written to both triangles. A block takes
+// one tile; group g of its eight groups of 64 threads adds the chunks g, g + 16, ..
+// and g + 8, g + 24, .. in two sums (eight loads before their adds), and the groups
+// are added in order.
+__global__ void __launch_bounds__(512)
+    k_gram_tri_reduce(const float* __restrict__ partial, int nchunks, int n, float* __restrict__ G) {
+  __shared__ float sums[8][64];
+  const int el = threadIdx.x & 63, grp = threadIdx.x >> 6, ng = (n + kG8 - 1) / kG8;
+  const int64_t stride = (int64_t)gridDim.x * 64;
+  const float* p = partial + (int64_t)blockIdx.x * 64 + el;
+  float s0 = 0.f, s1 = 0.f;
+  int ch = grp;
+  for (; ch + 56 < nchunks; ch += 64) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = __ldg(p + (int64_t)(ch + 8 * u) * stride);
+#pragma unroll
+    for (int u = 0; u < 8; u += 2) {
+      s0 += v[u];
+      s1 += v[u + 1];
+    }
+  }
+  for (; ch + 8 < nchunks; ch += 16) {
+    s0 += p[(int64_t)ch * stride];
+    s1 += p[(int64_t)(ch + 8) * stride];
+  }
+  if (ch < nchunks) s0 += p[(int64_t)ch * stride];
+  sums[grp][el] = s0 + s1;
+  __syncthreads();
+  if (grp) return;
+  int ti = 0, start = 0;
+  while (start + (ng - ti) <= (int)blockIdx.x) { start += ng - ti; ++ti; }
+  const int tj = ti + ((int)blockIdx.x - start);
+  const int a = ti * kG8 + (el >> 3), c = tj * kG8 + (el & 7);
+  if (a >= n || c >= n || (ti == tj && a > c)) return;
+  float t = 0.f;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) t += sums[g][el];
+  G[(int64_t)a * n + c] = t;
+  G[(int64_t)c * n + a] = t;
 }
 
 // G[e] = sum over chunks of the partial tiles. A block takes 32 consecutive
@@ -191,52 +319,194 @@ __global__ void __launch_bounds__(32 * kRedGroups)
 }
 
 // ---------------------------------------------------------------- X * T
-// Y[rows, 0:kout] = X[rows, map] T : 128-row x 128-column output tiles, the
-// inner dimension staged 16 at a time (X tile stored transposed so each
-// thread reads its 8 rows as two float4).
-__global__ void __launch_bounds__(256, 2)
-    k_gemm_ts(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
-              const float* __restrict__ T, int kout, float* __restrict__ Y, int ldy) {
-  __shared__ __align__(16) float Xs[kR][kT + 4];
-  __shared__ __align__(16) float Ts[kR][kT];
+// Y[rows, 0:kout] = X[rows, map] T, RT x 8 outputs per thread. A warp's lanes are 8 row
+// groups by 4 column groups (lane row lr of warp row wr has rows wr 8 RT + lr + 8 i),
+// so its loads of X and T from shared memory are one wavefront each, 16 per 4 inner
+// columns against 256 multiply-adds per lane at RT = 8. X and T arrive 16 inner
+// columns at a time through a ring of cp.async stages (T from L2), T's rows split in
+// halves as the Gram's. Each output adds its products in column order. Bound by the
+// packed multiply-adds where there are rows enough: 50,000 x 200 x 200 takes 131 us
+// (31 TFLOP/s; 205 in 128 x 128 tiles, where 200 columns left 28 % of a second tile's
+// work for padding), 20,000 x 100 x 100 27 us (46).
+constexpr int kMK = 16;        // inner columns per stage
+constexpr int kMLd = kMK + 4;  // X stage leading dimension: 8 rows start in 8 bank quads
+constexpr int kMStages = 3;
+constexpr int kMWideSmem = 226 * 1024;
+
+// acc += the stage's 16 inner columns: xs this lane's first row, tb its columns of T
+template <int RT>
+__device__ __forceinline__ void gemm_stage(float2 (&acc)[RT][4], const float* xs, const float* tb,
+                                           int ts, int ps) {
+#pragma unroll 1
+  for (int k = 0; k < kMK; k += 4) {
+    float4 a[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) a[i] = *reinterpret_cast<const float4*>(xs + i * 8 * kMLd + k);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float4 b0 = *reinterpret_cast<const float4*>(tb + (k + u) * ts);
+      const float4 b1 = *reinterpret_cast<const float4*>(tb + (k + u) * ts + ps);
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        const float x = u == 0 ? a[i].x : u == 1 ? a[i].y : u == 2 ? a[i].z : a[i].w;
+        pair_fma(acc[i][0], x, b0.x, b0.y);
+        pair_fma(acc[i][1], x, b0.z, b0.w);
+        pair_fma(acc[i][2], x, b1.x, b1.y);
+        pair_fma(acc[i][3], x, b1.z, b1.w);
+      }
+    }
+  }
+}
+
+// rows r0 + 8 i (< r_end) of this lane's column group tc
+template <int RT>
+__device__ __forceinline__ void gemm_store(const float2 (&acc)[RT][4], float* Y, int ldy, int64_t r0,
+                                           int64_t r_end, int tc, int kout, bool vec_y) {
+#pragma unroll
+  for (int i = 0; i < RT; ++i) {
+    const int64_t g = r0 + 8 * i;
+    if (g >= r_end) break;
+    float* y = Y + g * ldy + tc * 8;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 p = acc[i][2 * h], q = acc[i][2 * h + 1];
+      const int c = tc * 8 + 4 * h;
+      if (vec_y && c + 4 <= kout) {
+        *reinterpret_cast<float4*>(y + 4 * h) = make_float4(p.x, p.y, q.x, q.y);
+      } else {
+        if (c < kout) y[4 * h] = p.x;
+        if (c + 1 < kout) y[4 * h + 1] = p.y;
+        if (c + 2 < kout) y[4 * h + 2] = q.x;
+        if (c + 3 < kout) y[4 * h + 3] = q.y;
+      }
+    }
+  }
+}
+
+// row kk of T (zero past n rows and kout columns) by one warp, in copies of vec_t columns
+__device__ __forceinline__ void async_t_row(float* dst, const float* T, int kk, int n, int kout,
+                                            int wcols, int vec_t) {
+  const int ps = wcols * 16;
+  for (int c4 = threadIdx.x & 31; c4 < wcols * 8; c4 += 32) {
+    float* d = dst + (c4 & 1) * ps + (c4 >> 1) * 4;
+    const float* src = T + (int64_t)kk * kout + 4 * c4;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (t % vec_t) continue;
+      const bool ok = kk < n && 4 * c4 + t < kout;
+      if (vec_t == 4) async_copy16(d, ok ? src : T, ok ? 16 : 0);
+      else if (vec_t == 2) async_copy8(d + t, ok ? src + t : T, ok ? 8 : 0);
+      else async_copy4(d + t, ok ? src + t : T, ok);
+    }
+  }
+}
+
+template <int RT>
+__global__ void __launch_bounds__(512)
+    k_gemm_rows(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
+                const float* __restrict__ T, int kout, int wrows, int wcols, int vec_x, int vec_t,
+                bool vec_y, float* __restrict__ Y, int ldy) {
+  extern __shared__ __align__(16) float sm[];
   const int n = map.total();
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int64_t row0 = (int64_t)blockIdx.x * kT;
-  const int col0 = blockIdx.y * kT;
-  float acc[8][8] = {};
-  for (int c0 = 0; c0 < n; c0 += kR) {
+  const int ps = wcols * 16, ts = 2 * ps;  // T stage: half and whole row, in floats
+  const int xfl = wrows * 8 * RT * kMLd, stage = xfl + kMK * ts;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int r_lane = (warp / wcols) * 8 * RT + (lane >> 2), tc = (warp % wcols) * 4 + (lane & 3);
+  const int64_t row0 = (int64_t)blockIdx.x * wrows * 8 * RT;
+  const int nst = (n + kMK - 1) / kMK;
+  auto load = [&](int st) {
+    float* xs = sm + (st % kMStages) * stage;
+    float* tb = xs + xfl;
+    for (int i = tid; i < wrows * 8 * RT * (kMK / 4); i += blockDim.x) {
+      const int r = i >> 2, q = i & 3;
+      const int64_t g = row0 + r;
+      async_cols(xs + r * kMLd + 4 * q, X, ldx, map, g, st * (kMK / 4) + q, g < rows, vec_x);
+    }
+    for (int k = warp; k < kMK; k += nw)
+      async_t_row(tb + k * ts, T, st * kMK + k, n, kout, wcols, vec_t);
+  };
+  float2 acc[RT][4];
 #pragma unroll
-    for (int q = 0; q < (kT * kR) / 256; ++q) {
-      const int li = threadIdx.x + q * 256;
-      const int rr = li / kR, cc = li % kR;     // X tile: 128 rows x 16 inner
-      const int64_t g = row0 + rr;
-      const int c = c0 + cc;
-      Xs[cc][rr] = (g < rows && c < n) ? map.at(X, ldx, g, c) : 0.f;
-      const int tr = li / kT, tc = li % kT;     // T tile: 16 inner x 128 out
-      const int cr = c0 + tr, oc = col0 + tc;
-      Ts[tr][tc] = (cr < n && oc < kout) ? T[(int64_t)cr * kout + oc] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int cc = 0; cc < kR; ++cc) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&Xs[cc][ty * 8]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&Xs[cc][ty * 8 + 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Ts[cc][tx * 8]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Ts[cc][tx * 8 + 4]);
-      fma8x8(acc, a0, a1, b0, b1);
-    }
-    __syncthreads();
+  for (int i = 0; i < RT; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int st = 0; st < kMStages - 1; ++st) {
+    if (st < nst) load(st);
+    async_commit();
   }
+  for (int st = 0; st < nst; ++st) {
+    async_wait<kMStages - 2>();
+    __syncthreads();
+    if (st + kMStages - 1 < nst) load(st + kMStages - 1);
+    async_commit();
+    const float* xs = sm + (st % kMStages) * stage + r_lane * kMLd;
+    const float* tb = sm + (st % kMStages) * stage + xfl + tc * 4;
+    gemm_stage<RT>(acc, xs, tb, ts, ps);
+  }
+  async_wait<0>();
+  gemm_store<RT>(acc, Y, ldy, row0 + r_lane, rows, tc, kout, vec_y);
+}
+
+// The same product with T kept in shared memory (n kout up to about 46,000, 200 x 200
+// included): one CTA per SM, each with its own contiguous rows in tiles of wrows 8 RT,
+// so that only X moves during the products and the tiles of a CTA follow each other
+// through one ring of stages.
+template <int RT>
+__global__ void __launch_bounds__(512)
+    k_gemm_wide(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
+                int64_t rows_per_cta, const float* __restrict__ T, int kout, int wrows, int wcols,
+                int vec_x, int vec_t, bool vec_y, float* __restrict__ Y, int ldy) {
+  extern __shared__ __align__(16) float sm[];
+  const int n = map.total();
+  const int ps = wcols * 16, ts = 2 * ps;
+  const int nst = (n + kMK - 1) / kMK, tile = wrows * 8 * RT, xfl = tile * kMLd;
+  float* xbuf = sm + nst * kMK * ts;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int r_lane = (warp / wcols) * 8 * RT + (lane >> 2), tc = (warp % wcols) * 4 + (lane & 3);
+  const int64_t r_beg = (int64_t)blockIdx.x * rows_per_cta;
+  const int64_t r_end = min(rows, r_beg + rows_per_cta);
+  const int ntile = (int)((r_end - r_beg + tile - 1) / tile), total = ntile * nst;
+  auto load = [&](int s) {  // stage s % nst of tile s / nst
+    const int64_t row0 = r_beg + (int64_t)(s / nst) * tile;
+    float* xs = xbuf + (s % kMStages) * xfl;
+    for (int i = tid; i < tile * (kMK / 4); i += blockDim.x) {
+      const int r = i >> 2, q = i & 3;
+      async_cols(xs + r * kMLd + 4 * q, X, ldx, map, row0 + r, (s % nst) * (kMK / 4) + q,
+                 row0 + r < r_end, vec_x);
+    }
+  };
+  for (int k = warp; k < nst * kMK; k += nw) async_t_row(sm + k * ts, T, k, n, kout, wcols, vec_t);
+  float2 acc[RT][4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int64_t g = row0 + ty * 8 + i;
-    if (g >= rows) continue;
+  for (int i = 0; i < RT; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int oc = col0 + tx * 8 + j;
-      if (oc < kout) Y[g * ldy + oc] = acc[i][j];
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int s = 0; s < kMStages - 1; ++s) {  // T lands with the first stage
+    if (s < total) load(s);
+    async_commit();
+  }
+  int st = 0;  // stage within the tile
+  int64_t row0 = r_beg;
+  for (int s = 0; s < total; ++s) {
+    async_wait<kMStages - 2>();
+    __syncthreads();
+    if (s + kMStages - 1 < total) load(s + kMStages - 1);
+    async_commit();
+    gemm_stage<RT>(acc, xbuf + (s % kMStages) * xfl + r_lane * kMLd, sm + st * kMK * ts + tc * 4, ts,
+                   ps);
+    if (++st == nst) {
+      gemm_store<RT>(acc, Y, ldy, row0 + r_lane, r_end, tc, kout, vec_y);
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+      st = 0;
+      row0 += tile;
     }
   }
+  async_wait<0>();
 }
 
 // --------------------------------------------------- Cholesky + inverse
@@ -392,25 +662,49 @@ void launch_gauss_fill(float* out, int64_t rows, int cols, int ld, uint64_t seed
   SFD_LAUNCH_CHECK();
 }
 
+// columns per asynchronous copy: see async_cols
+static int vec_cols(const float* X, int ldx, const ColMap& map) {
+  for (int v = 4; v > 1; v >>= 1) {
+    const bool first = ldx % v == 0 && (uintptr_t)X % (4 * v) == 0;
+    if (first && (map.k1 == 0 || (map.k0 % v == 0 && map.ld1 % v == 0 &&
+                                  (uintptr_t)map.x1 % (4 * v) == 0)))
+      return v;
+  }
+  return 1;
+}
+
 void gram(const float* X, int ldx, ColMap map, int64_t rows, float* G, Workspace& ws,
           cudaStream_t s) {
-  const int n = map.total();
-  const int ntiles = (n + kT - 1) / kT;
-  const int npairs = ntiles * (ntiles + 1) / 2;
-  int nchunks = (int)std::max<int64_t>(1, std::min<int64_t>((rows + kR - 1) / kR, kGramBlocks / npairs));
+  const int n = map.total(), ng = (n + kG8 - 1) / kG8;
+  const int ntiles = ng * (ng + 1) / 2;
+  // chunks of rows and parts of the triangle: about two CTAs per SM. Rows are cut
+  // into the same chunks, and chunks added in the same order, as with 128 x 128 tiles,
+  // so a Gram keeps its bits; a chunk's tiles go to as many CTAs as it then had tiles.
+  const int n128 = (n + kT - 1) / kT, parts = n128 * (n128 + 1) / 2;
+  const int threads = ((ntiles + parts - 1) / parts + 31) & ~31;
+  int nchunks = (int)std::max<int64_t>(
+      1, std::min<int64_t>((rows + kGRows - 1) / kGRows, kGramBlocks / parts));
   int64_t rpc = (rows + nchunks - 1) / nchunks;
-  rpc = ((rpc + kR - 1) / kR) * kR;
+  rpc = ((rpc + kGRows - 1) / kGRows) * kGRows;
   nchunks = (int)std::max<int64_t>(1, (rows + rpc - 1) / rpc);
   float* partial = ws.gram_partial;
   if (rows > 0) {
-    dim3 grid(nchunks, npairs);
-    k_gram_tiles<<<grid, 256, 0, s>>>(X, ldx, map, rows, rpc, ntiles, npairs, partial);
+    const size_t bytes = (size_t)kGStages * kGRows * ng * kG8 * sizeof(float);
+    static std::atomic<unsigned> attr{0};
+    int dev = 0;
+    SFD_CUDA(cudaGetDevice(&dev));
+    if (dev < 32 && !(attr.load() & (1u << dev))) {
+      SFD_CUDA(cudaFuncSetAttribute(k_gram_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kGStages * kGRows * kMaxEig * (int)sizeof(float)));
+      attr.fetch_or(1u << dev);
+    }
+    k_gram_tri<<<dim3(nchunks, parts), threads, bytes, s>>>(X, ldx, map, rows, rpc, ntiles,
+                                                         vec_cols(X, ldx, map), partial);
     SFD_LAUNCH_CHECK();
   } else {
     nchunks = 0;
   }
-  int64_t ne = (int64_t)n * n;
-  k_gram_reduce<<<(unsigned)((ne + 31) / 32), 32 * kRedGroups, 0, s>>>(partial, nchunks, npairs, ntiles, n, G);
+  k_gram_tri_reduce<<<ntiles, 512, 0, s>>>(partial, nchunks, n, G);
   SFD_LAUNCH_CHECK();
 }
 
@@ -423,8 +717,54 @@ void gram_reduce_tiles(const float* partial, int nchunks, int n, float* G, cudaS
 void gemm_ts(const float* X, int ldx, ColMap map, int64_t rows, const float* T, int kout, float* Y,
              int ldy, cudaStream_t s) {
   if (rows <= 0 || kout <= 0) return;
-  dim3 grid((unsigned)((rows + kT - 1) / kT), (kout + kT - 1) / kT);
-  k_gemm_ts<<<grid, 256, 0, s>>>(X, ldx, map, rows, T, kout, Y, ldy);
+  const int wcols = (kout + 31) / 32;  // <= 8 (kout <= 256)
+  const int n = map.total();
+  const int vec_x = vec_cols(X, ldx, map);
+  int vec_t = 4;
+  while (vec_t > 1 && (kout % vec_t || (uintptr_t)T % (4 * vec_t))) vec_t >>= 1;
+  const bool vec_y = (ldy & 3) == 0 && ((uintptr_t)Y & 15) == 0;
+  static std::atomic<unsigned> attr{0};
+  int dev = 0;
+  SFD_CUDA(cudaGetDevice(&dev));
+  if (dev < 32 && !(attr.load() & (1u << dev))) {
+    for (auto f : {k_gemm_wide<4>, k_gemm_wide<5>, k_gemm_wide<6>, k_gemm_wide<7>, k_gemm_wide<8>})
+      SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMWideSmem));
+    const int most = kMStages * (128 * kMLd + kMK * kMaxEll) * (int)sizeof(float);
+    for (auto f : {k_gemm_rows<2>, k_gemm_rows<8>})
+      SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    attr.fetch_or(1u << dev);
+  }
+  // T in shared memory, one CTA per SM, where the rows fill the SMs (32 or more each):
+  // the rows per thread that waste least of the last tile
+  const size_t t_bytes = (size_t)((n + kMK - 1) / kMK) * kMK * wcols * 32 * sizeof(float);
+  const int wide_rows = std::max(1, 16 / wcols);
+  const size_t x_row = (size_t)kMStages * kMLd * sizeof(float);
+  if (rows >= 152 * 32 && t_bytes + wide_rows * 64 * x_row <= (size_t)kMWideSmem) {
+    const int64_t rpc = (rows + 151) / 152;
+    int rt = 8;
+    int64_t best = INT64_MAX;
+    for (int r = 8; r >= 4; --r) {
+      const int64_t cost = (rpc + wide_rows * 8 * r - 1) / (wide_rows * 8 * r) * r;
+      if (cost < best) {
+        best = cost;
+        rt = r;
+      }
+    }
+    auto k = rt == 8 ? k_gemm_wide<8> : rt == 7 ? k_gemm_wide<7> : rt == 6 ? k_gemm_wide<6>
+             : rt == 5 ? k_gemm_wide<5> : k_gemm_wide<4>;
+    k<<<(unsigned)((rows + rpc - 1) / rpc), wide_rows * wcols * 32,
+        t_bytes + wide_rows * 8 * rt * x_row, s>>>(X, ldx, map, rows, rpc, T, kout, wide_rows, wcols,
+                                                   vec_x, vec_t, vec_y, Y, ldy);
+    SFD_LAUNCH_CHECK();
+    return;
+  }
+  // else T through the stages: 64 rows per CTA (8 x 8 outputs per thread), 16 (2 x 8)
+  // where 64 would leave SMs without a CTA
+  const int rt = (rows + 63) / 64 < 2 * 152 ? 2 : 8, tile = 8 * rt;
+  const size_t bytes = (size_t)kMStages * (tile * kMLd + kMK * wcols * 32) * sizeof(float);
+  auto k = rt == 2 ? k_gemm_rows<2> : k_gemm_rows<8>;
+  k<<<(unsigned)((rows + tile - 1) / tile), wcols * 32, bytes, s>>>(
+      X, ldx, map, rows, T, kout, 1, wcols, vec_x, vec_t, vec_y, Y, ldy);
   SFD_LAUNCH_CHECK();
 }
 
