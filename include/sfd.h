@@ -201,7 +201,8 @@ const char* sfd_last_error(const sfd_ctx* ctx);
 /* ------------------------------------------------------------------------
  * One buffer / one stack (the per-step calls used to check each stage).
  * Device pointers only; the stream is the default stream of the calling
- * thread's current device. Each call allocates its own scratch.
+ * thread's current device. Scratch is kept between calls (512 MB at most) and
+ * freed by sfd_destroy, sfd_batch_destroy and when an allocation fails.
  * ------------------------------------------------------------------------ */
 
 /* BoostedSparseShrink (Alg. 4) of one buffer A' (m x d CSR with int32

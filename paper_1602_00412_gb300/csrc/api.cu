@@ -304,7 +304,7 @@ int sfd_create(int64_t d, int32_t ell, uint64_t seed, const sfd_options* opt, sf
     C.merger->mixed = C.opt.precision == 1;
     for (int i = 0; i < want; ++i) {
       try {
-        C.slots.emplace_back(new Slot(d, ell, d, cap_nnz, nullptr));
+        C.slots.emplace_back(new Slot(d, ell, d, cap_nnz));
         C.slots.back()->profile = C.opt.profile != 0;
         C.slots.back()->mixed = C.opt.precision == 1;
         C.slots.back()->autotune = C.opt.autotune != 0;
@@ -328,7 +328,10 @@ int sfd_create(int64_t d, int32_t ell, uint64_t seed, const sfd_options* opt, sf
   return SFD_OK;
 }
 
-void sfd_destroy(sfd_ctx* ctx) { delete ctx; }
+void sfd_destroy(sfd_ctx* ctx) {
+  delete ctx;
+  if (ctx) scratch_trim();
+}
 
 int sfd_append_rows(sfd_ctx* ctx, int64_t nrows, const int64_t* indptr, const int32_t* indices,
                     const float* values, int where) {
@@ -366,8 +369,8 @@ int sfd_append_rows(sfd_ctx* ctx, int64_t nrows, const int64_t* indptr, const in
         C.stage_idx = nullptr;
         C.stage_val = nullptr;
         C.stage_cap = 0;
-        SFD_CUDA(cudaMalloc(&C.stage_idx, total * sizeof(int)));
-        SFD_CUDA(cudaMalloc(&C.stage_val, total * sizeof(float)));
+        SFD_CUDA(device_malloc((void**)&C.stage_idx, total * sizeof(int)));
+        SFD_CUDA(device_malloc((void**)&C.stage_val, total * sizeof(float)));
         C.stage_cap = total;
       }
       if (total > 0) {

@@ -12,14 +12,14 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
+#include <new>
 
 #include "engine.cuh"
 
 namespace sfd {
 
 unsigned long long g_kernel_launches = 0;
-
-namespace {
 
 int bits_for(int64_t d) {
   int b = 1;
@@ -34,14 +34,162 @@ void alloc_work(DevArena& A, SegWork& w, int64_t nseg, int64_t nnz) {
   w.item_slot = A.alloc<int>(w.cap_items);
   w.item_split = A.alloc<int>(w.cap_items);
   w.split_ticket = A.alloc<unsigned>(w.cap_split);
-  SFD_CUDA(cudaMemset(w.split_ticket, 0, (size_t)w.cap_split * sizeof(unsigned)));
   w.split_seg = A.alloc<int>(std::max<int64_t>(nseg, 1) + 1);
   w.split_first = A.alloc<int>(std::max<int64_t>(nseg, 1) + 1);
   w.split_count = A.alloc<int>(std::max<int64_t>(nseg, 1) + 1);
   w.counters = A.alloc<int>(8 + 4 * ((size_t)nseg + 1) + nseg / 4096 + 16);
 }
 
+void clear_work(SegWork& w, cudaStream_t s) {
+  SFD_CUDA(cudaMemsetAsync(w.split_ticket, 0, (size_t)w.cap_split * sizeof(unsigned), s));
+}
+
+void alloc_sort(DevArena& A, SortBuffers& t, Workspace& ws, int64_t nnz, int64_t segs) {
+  t.key = A.alloc<int>(nnz);
+  t.key2 = A.alloc<int>(nnz);
+  t.a = A.alloc<int>(nnz);
+  t.b = A.alloc<float>(nnz);
+  const int64_t ntiles = (nnz + 4095) / 4096 + 1;
+  ws.hist_cap = (int)(512 * ntiles + 8);
+  ws.hist = A.alloc<int>(ws.hist_cap);
+  ws.scan_tmp = A.alloc<int>(std::max<int64_t>(ws.hist_cap, segs + 2) / 4096 + 64);
+}
+
+namespace {
+
+// idle scratches, the most recent last; guarded by g_scratch_m
+std::mutex g_scratch_m;
+Scratch* g_scratch_idle[kScratchIdle];
+int g_scratch_count = 0;
+
 }  // namespace
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    scratch_trim();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
+Scratch::Scratch() {
+  try {
+    SFD_CUDA(cudaGetDevice(&dev));
+    SFD_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
+    SFD_CUDA(cudaEventCreateWithFlags(&event, cudaEventDisableTiming));
+    void* p = nullptr;
+    const cudaError_t e = device_malloc(&p, 64 * sizeof(int));
+    if (e != cudaSuccess) throw CudaError{e, "cudaMalloc"};
+    head = static_cast<int*>(p);
+    SFD_CUDA(cudaMallocHost(&pinned, kScratchPinned));
+    if (!current_ctx_id(&ctx_id)) ctx_id = 0;
+  } catch (...) {
+    if (stream) cudaStreamDestroy(stream);
+    if (event) cudaEventDestroy(event);
+    if (head) cudaFree(head);
+    throw;
+  }
+}
+
+Scratch::~Scratch() {
+  cudaFree(block);
+  cudaFree(head);
+  cudaFreeHost(pinned);
+  cudaEventDestroy(event);
+  cudaStreamDestroy(stream);
+}
+
+char* Scratch::reserve(size_t n) {
+  if (n > bytes) {
+    cudaFree(block);
+    block = nullptr;
+    bytes = 0;
+    const size_t want = (n + ((size_t)2 << 20) - 1) & ~(((size_t)2 << 20) - 1);
+    void* p = nullptr;
+    const cudaError_t e = device_malloc(&p, want);
+    if (e != cudaSuccess) throw CudaError{e, "cudaMalloc"};
+    block = static_cast<char*>(p);
+    bytes = want;
+  }
+  return block;
+}
+
+ScratchLease::ScratchLease(bool all_streams) : s(nullptr) {
+  int dev = 0;
+  unsigned long long id = 0;
+  SFD_CUDA(cudaGetDevice(&dev));
+  SFD_CUDA(cudaFree(nullptr));  // the context exists from here on
+  if (!current_ctx_id(&id)) id = 0;
+  {
+    std::lock_guard<std::mutex> lock(g_scratch_m);
+    for (int i = g_scratch_count; i-- > 0 && !s;) {
+      Scratch* c = g_scratch_idle[i];
+      if (c->dev != dev) continue;
+      for (int j = i + 1; j < g_scratch_count; ++j) g_scratch_idle[j - 1] = g_scratch_idle[j];
+      --g_scratch_count;
+      if (c->ctx_id == id) s = c;
+      else ::operator delete(c);  // of a context that is gone, and its memory with it
+    }
+  }
+  if (!s) s = new Scratch();
+  try {
+    if (all_streams) {
+      SFD_CUDA(cudaDeviceSynchronize());
+    } else {
+      // An allocation is what CUDA refuses while a capture is under way whose work has
+      // not run yet (the input may be its output), so the call is refused then, also
+      // when its memory is there already; a small one takes 2 us.
+      void* probe = nullptr;
+      SFD_CUDA(cudaMalloc(&probe, 256));
+      SFD_CUDA(cudaFree(probe));
+      SFD_CUDA(cudaEventRecord(s->event, 0));
+      SFD_CUDA(cudaStreamWaitEvent(s->stream, s->event, 0));
+    }
+  } catch (...) {
+    delete s;
+    throw;
+  }
+}
+
+ScratchLease::~ScratchLease() {
+  bool keep = cudaStreamSynchronize(s->stream) == cudaSuccess && s->ctx_id != 0;
+  if (keep) {
+    std::lock_guard<std::mutex> lock(g_scratch_m);
+    size_t held = s->bytes;
+    for (int i = 0; i < g_scratch_count; ++i) held += g_scratch_idle[i]->bytes;
+    keep = g_scratch_count < kScratchIdle && held <= kScratchKeep;
+    if (keep) g_scratch_idle[g_scratch_count++] = s;
+  }
+  if (!keep) delete s;
+}
+
+void scratch_trim() {
+  Scratch* idle[kScratchIdle];
+  int n;
+  {
+    std::lock_guard<std::mutex> lock(g_scratch_m);
+    n = g_scratch_count;
+    std::copy(g_scratch_idle, g_scratch_idle + n, idle);
+    g_scratch_count = 0;
+  }
+  if (n == 0) return;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  for (int i = 0; i < n; ++i) {
+    unsigned long long id = 0;
+    cudaSetDevice(idle[i]->dev);
+    if (current_ctx_id(&id) && id == idle[i]->ctx_id) delete idle[i];
+    else ::operator delete(idle[i]);
+  }
+  cudaSetDevice(dev);
+}
+
+void clear_dense_scratch(Workspace& ws, cudaStream_t s) {
+  SFD_CUDA(cudaMemsetAsync(ws.scalars, 0, 64 * sizeof(double), s));
+  SFD_CUDA(cudaMemsetAsync(ws.flags, 0, 16 * sizeof(int), s));
+}
 
 void alloc_dense_scratch(DevArena& A, Workspace& ws) {
   ws.gram_partial = A.alloc<float>((size_t)320 * 128 * 128);
@@ -51,74 +199,79 @@ void alloc_dense_scratch(DevArena& A, Workspace& ws) {
   ws.eig_work = A.alloc<float>(symeig_work_floats(kMaxEig, kMaxEig));
   ws.scalars = A.alloc<double>(64);
   ws.flags = A.alloc<int>(16);
-  SFD_CUDA(cudaMemset(ws.scalars, 0, 64 * sizeof(double)));
-  SFD_CUDA(cudaMemset(ws.flags, 0, 16 * sizeof(int)));
 }
 
 // ======================================================================= Slot
-Slot::Slot(int64_t d_, int ell_, int64_t cap_rows_, int64_t cap_nnz_, cudaStream_t s) {
+Slot::Slot(int64_t d_, int ell_, int64_t cap_rows_, int64_t cap_nnz_, Scratch* from) {
   d = d_;
   ell = ell_;
   ld = ld_of(ell);
   cap_rows = std::max<int64_t>(cap_rows_, 1);
   cap_nnz = std::max<int64_t>(cap_nnz_, 1);
+  use_graphs = from == nullptr;
   try {
-    if (s) {
-      stream = s;
+    if (from) {
+      stream = from->stream;
     } else {
       SFD_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
       own_stream = true;
     }
     SFD_CUDA(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
     SFD_CUDA(cudaEventCreateWithFlags(&freed, cudaEventDisableTiming));
-    DevArena& A = arena;
-    csr.ptr = A.alloc<int>(cap_rows + 1);
-    csr.idx = A.alloc<int>(cap_nnz);
-    csr.val = A.alloc<float>(cap_nnz);
-    csc.ptr = A.alloc<int>(d + 1);
-    csc.idx = A.alloc<int>(cap_nnz);
-    csc.val = A.alloc<float>(cap_nnz);
-    key = A.alloc<int>(cap_nnz);
-    key2 = A.alloc<int>(cap_nnz);
-    a_alt = A.alloc<int>(cap_nnz);
-    b_alt = A.alloc<float>(cap_nnz);
-    alloc_work(A, csr.work, cap_rows, cap_nnz);
-    alloc_work(A, csc.work, d, cap_nnz);
     const size_t dense_d = (size_t)d * ld, dense_m = (size_t)cap_rows * ld;
-    W = A.alloc<float>(dense_d);
-    W2 = A.alloc<float>(dense_d);
-    Bpt = A.alloc<float>(dense_d);
-    Y = A.alloc<float>(dense_m);
-    Y2 = A.alloc<float>(dense_m);
-    Wh = A.alloc<__half>(dense_d);
-    Yh = A.alloc<__half>(dense_m);
-    SFD_CUDA(cudaMemset(Wh, 0, dense_d * sizeof(__half)));
-    SFD_CUDA(cudaMemset(Yh, 0, dense_m * sizeof(__half)));
-    for (float* p : {W, W2, Bpt}) SFD_CUDA(cudaMemset(p, 0, dense_d * sizeof(float)));
-    for (float* p : {Y, Y2}) SFD_CUDA(cudaMemset(p, 0, dense_m * sizeof(float)));
-    alloc_dense_scratch(A, ws);
-    int64_t ntiles = (cap_nnz + 4095) / 4096 + 1;
-    ws.hist_cap = (int)(512 * ntiles + 8);
-    ws.hist = A.alloc<int>(ws.hist_cap);
-    ws.scan_tmp = A.alloc<int>(std::max<int64_t>(ws.hist_cap, d + cap_rows + 2) / 4096 + 64);
-    int64_t slots = 2 * (cap_nnz / kSplit) + 4;
-    ws.partial_rows_cap = (int)slots;
-    ws.partial_rows = A.alloc<float>((size_t)slots * ld);
-    ws.vec0 = A.alloc<float>(d);
-    ws.vec1 = A.alloc<float>(std::max<int64_t>(d, cap_rows));
-    ws.vec2 = A.alloc<float>(d);
-    ws.wpart = A.alloc<float>(512 * kMaxEll + kMaxEll + 512);
-    fro2 = A.alloc<double>(1024 + 8);
-    verdict_dev = A.alloc<Verdict>(1);
-    qfeat = A.alloc<float>(kQF);
-    qacc = A.alloc<unsigned>(kQAccWords);
-    qy = A.alloc<float>(1);
-    q_dev = A.alloc<int>(1);
-    SFD_CUDA(cudaMallocHost(&verdict_host, sizeof(Verdict)));
-    SFD_CUDA(cudaMallocHost(&qfeat_host, kQF * sizeof(float)));
-    SFD_CUDA(cudaMallocHost(&q_host, sizeof(int)));
-    SFD_CUDA(cudaMallocHost(&ptr_host, (cap_rows + 1) * sizeof(int)));
-    SFD_CUDA(cudaDeviceSynchronize());
+    arena.carve(from, [&](DevArena& A) {
+      csr.ptr = A.alloc<int>(cap_rows + 1);
+      csr.idx = A.alloc<int>(cap_nnz);
+      csr.val = A.alloc<float>(cap_nnz);
+      csc.ptr = A.alloc<int>(d + 1);
+      csc.idx = A.alloc<int>(cap_nnz);
+      csc.val = A.alloc<float>(cap_nnz);
+      alloc_sort(A, sort, ws, cap_nnz, d + cap_rows);
+      alloc_work(A, csr.work, cap_rows, cap_nnz);
+      alloc_work(A, csc.work, d, cap_nnz);
+      W = A.alloc<float>(dense_d);
+      W2 = A.alloc<float>(dense_d);
+      Bpt = A.alloc<float>(dense_d);
+      Y = A.alloc<float>(dense_m);
+      Y2 = A.alloc<float>(dense_m);
+      Wh = A.alloc<__half>(dense_d);
+      Yh = A.alloc<__half>(dense_m);
+      alloc_dense_scratch(A, ws);
+      int64_t slots = 2 * (cap_nnz / kSplit) + 4;
+      ws.partial_rows_cap = (int)slots;
+      ws.partial_rows = A.alloc<float>((size_t)slots * ld);
+      ws.vec0 = A.alloc<float>(d);
+      ws.vec1 = A.alloc<float>(std::max<int64_t>(d, cap_rows));
+      ws.vec2 = A.alloc<float>(d);
+      ws.wpart = A.alloc<float>(512 * kMaxEll + kMaxEll + 512);
+      fro2 = A.alloc<double>(1024 + 8);
+      verdict_dev = A.alloc<Verdict>(1);
+      qfeat = A.alloc<float>(kQF);
+      qacc = A.alloc<unsigned>(kQAccWords);
+      qy = A.alloc<float>(1);
+      q_dev = A.alloc<int>(1);
+    });
+    SFD_CUDA(cudaMemsetAsync(Wh, 0, dense_d * sizeof(__half), stream));
+    SFD_CUDA(cudaMemsetAsync(Yh, 0, dense_m * sizeof(__half), stream));
+    for (float* p : {W, W2, Bpt}) SFD_CUDA(cudaMemsetAsync(p, 0, dense_d * sizeof(float), stream));
+    for (float* p : {Y, Y2}) SFD_CUDA(cudaMemsetAsync(p, 0, dense_m * sizeof(float), stream));
+    for (Csr* c : {&csr, &csc}) clear_work(c->work, stream);
+    clear_dense_scratch(ws, stream);
+    // pinned: verdict, features, power count, then (a context's slot) the row pointer
+    const size_t small = 1024;
+    char* h;
+    if (from) {
+      h = from->pinned;
+    } else {
+      SFD_CUDA(cudaMallocHost(&pinned, small + (cap_rows + 1) * sizeof(int)));
+      h = static_cast<char*>(pinned);
+      ptr_host = reinterpret_cast<int*>(h + small);
+    }
+    verdict_host = reinterpret_cast<Verdict*>(h);
+    qfeat_host = reinterpret_cast<float*>(h + 256);
+    q_host = reinterpret_cast<int*>(h + 512);
+    static_assert(sizeof(Verdict) <= 256 && kQF * sizeof(float) <= 256, "pinned layout");
+    if (!from) SFD_CUDA(cudaStreamSynchronize(stream));
   } catch (...) {
     cleanup();
     throw;
@@ -137,10 +290,8 @@ void Slot::cleanup() {
     }
   vs_graphs.release();
   arena.release();
-  if (verdict_host) cudaFreeHost(verdict_host);
-  if (ptr_host) cudaFreeHost(ptr_host);
-  if (qfeat_host) cudaFreeHost(qfeat_host);
-  if (q_host) cudaFreeHost(q_host);
+  if (pinned) cudaFreeHost(pinned);
+  pinned = nullptr;
   verdict_host = nullptr;
   ptr_host = nullptr;
   qfeat_host = nullptr;
@@ -165,16 +316,22 @@ void Slot::build(int m, int64_t nnz, int64_t max_row) {
   csr.may_split = max_row < 0 || max_row > kSplit;
   launch_check_entries(csr.idx, csr.val, nnz, (int)d, nullptr, fro2, ws.flags, stream);
   build_work(csr, stream);
-  // CSC by a stable radix sort of (col, row, val) by col
-  SFD_CUDA(cudaMemcpyAsync(key, csr.idx, nnz * sizeof(int), cudaMemcpyDeviceToDevice, stream));
-  SFD_CUDA(cudaMemcpyAsync(csc.val, csr.val, nnz * sizeof(float), cudaMemcpyDeviceToDevice, stream));
-  launch_row_ids(csr.ptr, m, csc.idx, stream);
-  radix_sort_by_key(key, csc.idx, csc.val, key2, a_alt, b_alt, nnz, bits_for(d), ws.hist,
-                    ws.scan_tmp, stream);
-  colptr_from_sorted(key, nnz, (int)d, csc.ptr, stream);
-  csc.nseg = (int)d;
+  build_csc(csr, csc, (int)d, sort, ws, stream);
+}
+
+// by a stable radix sort of (col, row, val) by col
+void build_csc(const Csr& csr, Csr& csc, int d, const SortBuffers& t, const Workspace& ws,
+               cudaStream_t s) {
+  const int64_t nnz = csr.nnz;
+  SFD_CUDA(cudaMemcpyAsync(t.key, csr.idx, nnz * sizeof(int), cudaMemcpyDeviceToDevice, s));
+  SFD_CUDA(cudaMemcpyAsync(csc.val, csr.val, nnz * sizeof(float), cudaMemcpyDeviceToDevice, s));
+  launch_row_ids(csr.ptr, csr.nseg, csc.idx, s);
+  radix_sort_by_key(t.key, csc.idx, csc.val, t.key2, t.a, t.b, nnz, bits_for(d), ws.hist,
+                    ws.scan_tmp, s);
+  colptr_from_sorted(t.key, nnz, d, csc.ptr, s);
+  csc.nseg = d;
   csc.nnz = nnz;
-  build_work(csc, stream);
+  build_work(csc, s);
 }
 
 bool Slot::orth_pass(const float* X, int64_t rows, float* Xout, int form, __half* Xh) {
@@ -324,7 +481,7 @@ int Slot::enqueue_attempt(int m, int q, uint64_t seed, uint64_t b, uint64_t r, i
   launch_delta(fro2, ws.scalars, ell, stream);
   if (verify) {
     VsArgs a{&csr, &csc, Bpt, ld, ell, d, m, ws.scalars + kSscale, p, seed, b, r};
-    verify_spectral(a, ws, stream, &vs_graphs);
+    verify_spectral(a, ws, stream, use_graphs ? &vs_graphs : nullptr);
   }
   launch_verdict(fro2, ws.scalars, ws.flags, ws.evals, ell, verify, verdict_dev, stream);
   SFD_CUDA(cudaMemcpyAsync(verdict_host, verdict_dev, sizeof(Verdict), cudaMemcpyDeviceToHost,
@@ -334,17 +491,26 @@ int Slot::enqueue_attempt(int m, int q, uint64_t seed, uint64_t b, uint64_t r, i
 }
 
 // ===================================================================== Merger
-Merger::Merger(int64_t d_, int ell_) {
+Merger::Merger(int64_t d_, int ell_, Scratch* from) {
   d = d_;
   ell = ell_;
   ld = ld_of(ell);
   try {
-    SFD_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
-    for (int i = 0; i < 2; ++i) Bt[i] = arena.alloc<float>((size_t)d * ld);
-    out = arena.alloc<float>((size_t)d * ell);
-    alloc_dense_scratch(arena, ws);
+    if (from) {
+      stream = from->stream;
+    } else {
+      SFD_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
+      own_stream = true;
+    }
+    arena.carve(from, [&](DevArena& A) {
+      for (int i = 0; i < 2; ++i) Bt[i] = A.alloc<float>((size_t)d * ld);
+      out = A.alloc<float>((size_t)d * std::max(ell, ld));
+      if (from) stack = A.alloc<float>((size_t)d * ld);
+      alloc_dense_scratch(A, ws);
+    });
+    clear_dense_scratch(ws, stream);
     zero();
-    SFD_CUDA(cudaStreamSynchronize(stream));
+    if (!from) SFD_CUDA(cudaStreamSynchronize(stream));
   } catch (...) {
     cleanup();
     throw;
@@ -355,7 +521,7 @@ Merger::~Merger() { cleanup(); }
 
 void Merger::cleanup() {
   arena.release();
-  if (stream) cudaStreamDestroy(stream);
+  if (own_stream && stream) cudaStreamDestroy(stream);
   stream = nullptr;
 }
 

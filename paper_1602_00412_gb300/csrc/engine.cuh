@@ -15,32 +15,129 @@
 // to pinned host memory at the end of an attempt.
 #pragma once
 
+#include <algorithm>
 #include <vector>
 
 #include "sfd_internal.cuh"
 
 namespace sfd {
 
-// Device allocations of one owner, freed together.
+// What a one-shot call works in: a stream, a block of device memory, pinned memory
+// and an event. Creating and freeing these cost several times the kernels of most
+// calls (a Gram of 50,000 x 100: 274 us a call, 20 us of kernels; 43 us a call now), so a finished call
+// leaves them to the next one. A call holds its Scratch alone, whatever its thread or
+// stream. At most kScratchIdle idle ones of kScratchKeep bytes together are kept, each
+// for its own CUDA context; they are freed when an allocation of the library fails and
+// when a context (sfd_destroy) or a batch is destroyed.
+constexpr int kScratchIdle = 4;
+constexpr size_t kScratchKeep = (size_t)512 << 20;
+constexpr size_t kScratchPinned = 4096;
+
+struct Scratch {
+  int dev = 0;
+  unsigned long long ctx_id = 0;
+  cudaStream_t stream = nullptr;
+  cudaEvent_t event = nullptr;
+  char* block = nullptr;
+  size_t bytes = 0;
+  char* pinned = nullptr;
+  int* head = nullptr;  // 64 device ints beside the block
+
+  Scratch();
+  ~Scratch();
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
+  char* reserve(size_t n);  // a block of at least n bytes; its contents are not kept
+};
+// A Scratch for the time of one call, its stream ordered after the caller's legacy
+// default stream (all_streams: after everything queued on the device). The stream is
+// synchronised before the Scratch is given back.
+struct ScratchLease {
+  Scratch* s;
+  explicit ScratchLease(bool all_streams = false);
+  ~ScratchLease();
+  ScratchLease(const ScratchLease&) = delete;
+  ScratchLease& operator=(const ScratchLease&) = delete;
+  Scratch* operator->() { return s; }
+};
+void scratch_trim();  // free the idle ones of every thread
+// cudaMalloc; on failure once more after scratch_trim
+cudaError_t device_malloc(void** p, size_t bytes);
+// Id of the calling thread's current CUDA context (0 when there is none).
+bool current_ctx_id(unsigned long long* id);
+
+// Device memory of one owner. Its layout is run twice, first to measure (alloc gives
+// null), then to carve one block: its own, or a Scratch's. What is allocated later
+// and does not fit the block gets its own cudaMalloc. All of it is freed together.
 struct DevArena {
   std::vector<void*> ptrs;
+  char* base = nullptr;
+  size_t off = 0, cap = 0;
+  bool measuring = false;
+  static size_t rounded(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
   template <typename T>
   T* alloc(size_t n) {
+    const size_t need = rounded(std::max<size_t>(n, 1) * sizeof(T));
+    if (measuring) {
+      off += need;
+      return nullptr;
+    }
+    if (base && off + need <= cap) {
+      T* p = reinterpret_cast<T*>(base + off);
+      off += need;
+      return p;
+    }
     void* p = nullptr;
-    if (n == 0) n = 1;
-    cudaError_t e = cudaMalloc(&p, n * sizeof(T));
+    cudaError_t e = device_malloc(&p, need);
     if (e != cudaSuccess) throw CudaError{e, "cudaMalloc"};
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
+  // run layout(*this) over one block for everything it allocates
+  template <typename F>
+  void carve(Scratch* from, F&& layout) {
+    measuring = true;
+    off = 0;
+    layout(*this);
+    measuring = false;
+    const size_t total = off;
+    if (from) {
+      base = from->reserve(total);
+    } else {
+      void* p = nullptr;
+      cudaError_t e = device_malloc(&p, total);
+      if (e != cudaSuccess) throw CudaError{e, "cudaMalloc"};
+      ptrs.push_back(p);
+      base = static_cast<char*>(p);
+    }
+    off = 0;
+    cap = total;
+    layout(*this);
+  }
   void release() {
     for (void* p : ptrs) cudaFree(p);
     ptrs.clear();
+    base = nullptr;
+    off = cap = 0;
   }
 };
 
-// Scratch of the dense stages (Gram, Cholesky, eigensolver, weights).
+// Scratch of the dense stages (Gram, Cholesky, eigensolver, weights); its status
+// words start at zero (clear_dense_scratch).
 void alloc_dense_scratch(DevArena& A, Workspace& ws);
+void clear_dense_scratch(Workspace& ws, cudaStream_t s);
+// Work lists of up to nseg segments and nnz entries (tickets zeroed by clear_work),
+// and the scratch of the radix sort and scans.
+void alloc_work(DevArena& A, SegWork& w, int64_t nseg, int64_t nnz);
+void clear_work(SegWork& w, cudaStream_t s);
+struct SortBuffers {  // ping-pong arrays of the radix sort
+  int *key = nullptr, *key2 = nullptr, *a = nullptr;
+  float* b = nullptr;
+};
+void alloc_sort(DevArena& A, SortBuffers& t, Workspace& ws, int64_t nnz, int64_t segs);
+// csc (allocated) of the columns of csr, and its work list
+void build_csc(const Csr& csr, Csr& csc, int d, const SortBuffers& t, const Workspace& ws,
+               cudaStream_t s);
 
 // How an attempt chooses its power count (the learned form; Alg. 1's q).
 struct QControl {
@@ -61,15 +158,15 @@ struct Slot {
   bool freed_pending = false;   // `freed` has been recorded and not yet waited on
   DevArena arena;
   Csr csr, csc;
-  int *key = nullptr, *key2 = nullptr, *a_alt = nullptr;
-  float* b_alt = nullptr;
+  SortBuffers sort;
   float *W = nullptr, *W2 = nullptr, *Y = nullptr, *Y2 = nullptr;
   __half *Wh = nullptr, *Yh = nullptr;  // fp16 copies of orthonormal blocks (mixed precision)
   float* Bpt = nullptr;         // B'^T, d x ld
   Workspace ws;
   double* fro2 = nullptr;       // [0] ||A'||_F^2, [1..] partials
   Verdict* verdict_dev = nullptr;
-  Verdict* verdict_host = nullptr;  // pinned
+  Verdict* verdict_host = nullptr;  // pinned, as the other _host pointers
+  void* pinned = nullptr;           // their memory, when it is the slot's own
   // learned q: features and prediction of the current buffer
   float* qfeat = nullptr;           // device, kQF
   unsigned* qacc = nullptr;         // device, kQAccWords
@@ -91,6 +188,7 @@ struct Slot {
   int (*choice)[2] = spmm_choice;
   cudaEvent_t tune_ev[2] = {nullptr, nullptr};
   VsGraphs vs_graphs;  // VerifySpectral steps, captured on first use
+  bool use_graphs = true;  // false in a one-shot call: one replay does not repay a capture
   // profiling of the sparse products
   bool profile = false;
   std::vector<cudaEvent_t> ev_pool;
@@ -99,7 +197,8 @@ struct Slot {
   int64_t prof_launches = 0;
   double prof_ms = 0, prof_bytes = 0;
 
-  Slot(int64_t d, int ell, int64_t cap_rows, int64_t cap_nnz, cudaStream_t s);
+  // from: run on this Scratch's stream and memory (a one-shot call); null: own both
+  Slot(int64_t d, int ell, int64_t cap_rows, int64_t cap_nnz, Scratch* from = nullptr);
   ~Slot();
   Slot(const Slot&) = delete;
   Slot& operator=(const Slot&) = delete;
@@ -135,13 +234,15 @@ struct Merger {
   int64_t d = 0;
   int ell = 0, ld = 0;
   cudaStream_t stream = nullptr;
+  bool own_stream = false;
   DevArena arena;
   float* Bt[2] = {nullptr, nullptr};  // d x ld
   float* out = nullptr;               // l x d: the sketch, transposed for a host copy
+  float* stack = nullptr;             // d x ld: a one-shot call's second block
   int cur = 0;
   Workspace ws;
 
-  Merger(int64_t d, int ell);
+  Merger(int64_t d, int ell, Scratch* from = nullptr);
   ~Merger();
   Merger(const Merger&) = delete;
   Merger& operator=(const Merger&) = delete;

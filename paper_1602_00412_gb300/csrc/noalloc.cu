@@ -19,7 +19,7 @@
 
 #include <mutex>
 
-#include "sfd_internal.cuh"
+#include "engine.cuh"
 
 namespace sfd {
 namespace {
@@ -53,6 +53,8 @@ std::mutex g_mu;
 using CtxGetCurrent = CUresult (*)(CUcontext*);
 using CtxGetId = CUresult (*)(CUcontext, unsigned long long*);
 
+}  // namespace
+
 // Id of the calling thread's current context (0 when there is none).
 bool current_ctx_id(unsigned long long* id) {
   static CtxGetCurrent get_current = nullptr;
@@ -75,6 +77,8 @@ bool current_ctx_id(unsigned long long* id) {
   *id = 0;
   return !ctx || get_id(ctx, id) == CUDA_SUCCESS;
 }
+
+namespace {
 
 // Device address of g_symeig_scratch in the current context of device `dev`,
 // resolved by cudaGetSymbolAddress once per device and context (with that
