@@ -73,13 +73,15 @@ __global__ void k_gauss_fill(float* __restrict__ out, int64_t rows, int cols, in
 // ------------------------------------------------------------------ Gram
 // 8 x 8 register tiles of the upper triangle of G, one per thread: 7 (7 + 1) / 2 = 28
 // of them for n = 50, 325 for n = 200, where 128 x 128 tiles computed 2.4 times as many
-// products. Rows arrive 16 at a time through a ring of cp.async
-// stages. A row of a stage holds the first four columns of every group of eight, then
-// the second four, so that neighbouring tiles' float4 loads use different banks. The
-// multiply-adds are packed two columns at a time (half the issue slots; each is rounded
-// as fmaf) and bound the kernel: 64 per thread and row against 4 shared float4 loads.
-// Cold, with its reduction: 100,000 x 200 127 us (31 TFLOP/s over both triangles; 438 in
-// 128 x 128 tiles), 20,000 x 100 27 us (49), 2,000 x 50 12 us.
+// products. Tile column g of ng stands for columns 4 g .. 4 g + 3 and 4 (ng + g) ..
+// 4 (ng + g) + 3, so that neighbouring tiles' float4 loads use different banks with the
+// rows as they lie in memory. Rows arrive 16 at a time through a ring of cp.async
+// stages, as a straight copy where rows are contiguous (k_gram_tri). The multiply-adds
+// are packed two columns at a time (half the issue slots; each is rounded as fmaf) and
+// bound the kernel: 64 per thread and row against 4 shared float4 loads.
+// Cold, with its reduction: 100,000 x 200 128 us (31 TFLOP/s counting both triangles; 438
+// in 128 x 128 tiles, 168 with row by row copies), 20,000 x 100 23 us (49, 25), 2,000 x
+// 50 11 us (15 with row by row copies).
 constexpr int kT = 128;  // output tile of the tensor-core Grams' partials
 constexpr int kG8 = 8;
 constexpr int kGRows = 16;    // rows per stage
@@ -146,12 +148,18 @@ __device__ __forceinline__ void async_cols(float* dst, const float* X, int ldx, 
 }
 
 // partial[chunk][tile][64]: tiles of the upper triangle in row-major order.
+// pitch: floats between rows, of both blocks, when a stage is 16 pitch floats of each
+// block as they lie (both start on 16 bytes, pitch and the first block's width are
+// multiples of 4): a float4 per thread and step, 6 instructions each where the row by
+// row copies of pitch = 0 need 25 and took as long as the products.
 __global__ void __launch_bounds__(512)
     k_gram_tri(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
-               int64_t rows_per_chunk, int ntiles, int vec, float* __restrict__ partial) {
+               int64_t rows_per_chunk, int ntiles, int vec, int pitch, float* __restrict__ partial) {
   extern __shared__ __align__(16) float sm[];
   const int n = map.total(), ng = (n + kG8 - 1) / kG8;
-  const int rs = ng * kG8, ps = ng * 4;  // floats per row and per half of it
+  const int rs = pitch ? pitch : ng * kG8;  // floats between rows of a stage
+  const int split = pitch && map.k1 ? kGRows * rs : 0;  // where its second block begins
+  const int stage = split ? 2 * split : kGRows * rs;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int slot = (int)(blockIdx.y * blockDim.x) + tid, e = min(slot, ntiles - 1);
   int ti = 0, start = 0;
@@ -162,15 +170,39 @@ __global__ void __launch_bounds__(512)
     while (start + (ng - ti) <= e) { start += ng - ti; ++ti; }
   }
   const int tj = ti + (e - start);
+  // offset in a stage of columns 4 q .. 4 q + 3 (of the last ones when there are none:
+  // those products are dropped, as those of columns past n are)
+  auto quad = [&](int q) {
+    const int c = 4 * min(q, (n - 1) >> 2);
+    return split && c >= map.k0 ? split + c - map.k0 : c;
+  };
+  const int qa = quad(ti), qb = quad(ng + ti), qc = quad(tj), qd = quad(ng + tj);
   const int64_t r_beg = (int64_t)blockIdx.x * rows_per_chunk;
   const int64_t r_end = min(rows, r_beg + rows_per_chunk);
   const int nst = (int)((r_end - r_beg + kGRows - 1) / kGRows);
   auto load = [&](int st) {
-    float* buf = sm + (st % kGStages) * kGRows * rs;
-    for (int r = warp; r < kGRows; r += nw) {
-      const int64_t g = r_beg + (int64_t)st * kGRows + r;
-      for (int c4 = lane; c4 < 2 * ng; c4 += 32)
-        async_cols(buf + r * rs + (c4 & 1) * ps + (c4 >> 1) * 4, X, ldx, map, g, c4, g < r_end, vec);
+    float* buf = sm + (st % kGStages) * stage;
+    const int64_t r0 = r_beg + (int64_t)st * kGRows;
+    if (pitch) {
+      const int before = ((int)min((int64_t)kGRows, r_end - r0) - 1) * rs;  // the last row
+      const float* src = X + r0 * ldx;
+      const int valid = before + map.k0;
+      for (int i = 4 * tid; i < kGRows * rs; i += 4 * blockDim.x) {
+        const int w = max(0, min(4, valid - i));
+        async_copy16(buf + i, w ? src + i : X, 4 * w);
+      }
+      if (split) {
+        const float* src1 = map.x1 + r0 * map.ld1;
+        const int valid1 = before + map.k1;
+        for (int i = 4 * tid; i < kGRows * rs; i += 4 * blockDim.x) {
+          const int w = max(0, min(4, valid1 - i));
+          async_copy16(buf + split + i, w ? src1 + i : X, 4 * w);
+        }
+      }
+    } else {
+      for (int r = warp; r < kGRows; r += nw)
+        for (int c4 = lane; c4 < 2 * ng; c4 += 32)
+          async_cols(buf + r * rs + 4 * c4, X, ldx, map, r0 + r, c4, r0 + r < r_end, vec);
     }
   };
   float2 acc[8][4];
@@ -188,15 +220,15 @@ __global__ void __launch_bounds__(512)
     __syncthreads();  // stage st has landed, and everyone is done with stage st - 1
     if (st + kGStages - 1 < nst) load(st + kGStages - 1);
     async_commit();
-    const float* buf = sm + (st % kGStages) * kGRows * rs;
+    const float* buf = sm + (st % kGStages) * stage;
     // the next row's operands are on their way while this row's products are formed
     float4 f[2][4];
     auto fetch = [&](int r, float4 (&q)[4]) {
       const float* row = buf + r * rs;
-      q[0] = *reinterpret_cast<const float4*>(row + ti * 4);
-      q[1] = *reinterpret_cast<const float4*>(row + ps + ti * 4);
-      q[2] = *reinterpret_cast<const float4*>(row + tj * 4);
-      q[3] = *reinterpret_cast<const float4*>(row + ps + tj * 4);
+      q[0] = *reinterpret_cast<const float4*>(row + qa);
+      q[1] = *reinterpret_cast<const float4*>(row + qb);
+      q[2] = *reinterpret_cast<const float4*>(row + qc);
+      q[3] = *reinterpret_cast<const float4*>(row + qd);
     };
     fetch(0, f[0]);
 #pragma unroll 2
@@ -256,7 +288,8 @@ __global__ void __launch_bounds__(512)
   int ti = 0, start = 0;
   while (start + (ng - ti) <= (int)blockIdx.x) { start += ng - ti; ++ti; }
   const int tj = ti + ((int)blockIdx.x - start);
-  const int a = ti * kG8 + (el >> 3), c = tj * kG8 + (el & 7);
+  auto col = [&](int g, int i) { return i < 4 ? 4 * g + i : 4 * (ng + g) + i - 4; };
+  const int a = col(ti, el >> 3), c = col(tj, el & 7);
   if (a >= n || c >= n || (ti == tj && a > c)) return;
   float t = 0.f;
 #pragma unroll
@@ -326,8 +359,8 @@ __global__ void __launch_bounds__(32 * kRedGroups)
 // columns at a time through a ring of cp.async stages (T from L2), T's rows split in
 // halves as the Gram's. Each output adds its products in column order. Bound by the
 // packed multiply-adds where there are rows enough: 50,000 x 200 x 200 takes 131 us
-// (31 TFLOP/s; 205 in 128 x 128 tiles, where 200 columns left 28 % of a second tile's
-// work for padding), 20,000 x 100 x 100 27 us (46).
+// (31 TFLOP/s; 205 in 128 x 128 tiles, a fifth of their products padding), 20,000 x 100
+// x 100 27 us (46).
 constexpr int kMK = 16;        // inner columns per stage
 constexpr int kMLd = kMK + 4;  // X stage leading dimension: 8 rows start in 8 bank quads
 constexpr int kMStages = 3;
@@ -689,17 +722,22 @@ void gram(const float* X, int ldx, ColMap map, int64_t rows, float* G, Workspace
   nchunks = (int)std::max<int64_t>(1, (rows + rpc - 1) / rpc);
   float* partial = ws.gram_partial;
   if (rows > 0) {
-    const size_t bytes = (size_t)kGStages * kGRows * ng * kG8 * sizeof(float);
+    const int vec = vec_cols(X, ldx, map);
+    // straight copies where little of a row is padding
+    const bool straight = vec == 4 && ldx <= ng * kG8 && (map.k1 == 0 || map.ld1 == ldx);
+    const int pitch = straight ? ldx : 0;
+    const int row = straight ? (map.k1 ? 2 : 1) * ldx : ng * kG8;
+    const size_t bytes = (size_t)kGStages * kGRows * row * sizeof(float);
     static std::atomic<unsigned> attr{0};
     int dev = 0;
     SFD_CUDA(cudaGetDevice(&dev));
     if (dev < 32 && !(attr.load() & (1u << dev))) {
       SFD_CUDA(cudaFuncSetAttribute(k_gram_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kGStages * kGRows * kMaxEig * (int)sizeof(float)));
+                                    2 * kGStages * kGRows * kMaxEig * (int)sizeof(float)));
       attr.fetch_or(1u << dev);
     }
-    k_gram_tri<<<dim3(nchunks, parts), threads, bytes, s>>>(X, ldx, map, rows, rpc, ntiles,
-                                                         vec_cols(X, ldx, map), partial);
+    k_gram_tri<<<dim3(nchunks, parts), threads, bytes, s>>>(X, ldx, map, rows, rpc, ntiles, vec,
+                                                            pitch, partial);
     SFD_LAUNCH_CHECK();
   } else {
     nchunks = 0;
@@ -734,8 +772,9 @@ void gemm_ts(const float* X, int ldx, ColMap map, int64_t rows, const float* T, 
       SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     attr.fetch_or(1u << dev);
   }
-  // T in shared memory, one CTA per SM, where the rows fill the SMs (32 or more each):
-  // the rows per thread that waste least of the last tile
+  // T in shared memory, one CTA per SM, where the rows fill the SMs (32 or more each; 130
+  // against 180 us through the stages at 50,000 x 200 x 200, 24 against 36 at 10,000 x
+  // 100 x 100), with the rows per thread that waste least of the last tile
   const size_t t_bytes = (size_t)((n + kMK - 1) / kMK) * kMK * wcols * 32 * sizeof(float);
   const int wide_rows = std::max(1, 16 / wcols);
   const size_t x_row = (size_t)kMStages * kMLd * sizeof(float);
