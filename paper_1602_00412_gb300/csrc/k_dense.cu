@@ -481,6 +481,93 @@ __global__ void __launch_bounds__(512)
   gemm_store<RT>(acc, Y, ldy, row0 + r_lane, rows, tc, kout, vec_y);
 }
 
+// The same product for few rows, where a call is one chain of latencies: T and 16 rows
+// of X arrive as they lie in memory, in one round of straight copies (no stages, no
+// arithmetic per element), then each thread forms 2 x 4 outputs. X as k_gram_tri's
+// straight copies want it, T on 16 bytes; VT is the width of T's shared loads (4, 2
+// or 1, a divisor of kout).
+// Cold: 2,000 x 50 x 50 7.7 us (18 through the stages), 4,800 x 100 x 100 10 (22),
+// 4,000 x 200 x 200 24 (43).
+constexpr int kSRows = 16;
+
+template <int VT>
+__global__ void __launch_bounds__(512)
+    k_gemm_small(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
+                 const float* __restrict__ T, int kout, bool vec_y, float* __restrict__ Y, int ldy) {
+  extern __shared__ __align__(16) float sm[];
+  const int n = map.total(), tid = threadIdx.x;
+  const int t_floats = (n * kout + 7) & ~3;  // the last row's unused columns included
+  float* xs = sm + t_floats;
+  const int split = map.k1 ? kSRows * ldx : 0;
+  const int64_t row0 = (int64_t)blockIdx.x * kSRows;
+  const int before = ((int)min((int64_t)kSRows, rows - row0) - 1) * ldx;
+  const int valid = before + map.k0, valid1 = before + map.k1, t_valid = n * kout;
+  const float* src = X + row0 * ldx;
+  for (int i = 4 * tid; i < kSRows * ldx; i += 4 * blockDim.x) {
+    const int w = max(0, min(4, valid - i));
+    async_copy16(xs + i, w ? src + i : X, 4 * w);
+    if (split) {
+      const int w1 = max(0, min(4, valid1 - i));
+      async_copy16(xs + split + i, w1 ? map.x1 + row0 * ldx + i : X, 4 * w1);
+    }
+  }
+  for (int i = 4 * tid; i < t_floats; i += 4 * blockDim.x) {
+    const int w = max(0, min(4, t_valid - i));
+    async_copy16(sm + i, w ? T + i : T, 4 * w);
+  }
+  async_commit();
+  async_wait<0>();
+  __syncthreads();
+  const int groups = (kout + 3) >> 2;
+  if (tid >= groups * (kSRows / 2)) return;
+  const int c = 4 * (tid % groups), r = 2 * (tid / groups);
+  float2 acc[2][2] = {};
+  const float* x0 = xs + r * ldx;
+  const float* tc = sm + c;
+  auto step = [&](float a0, float a1, int k) {
+    const float* t = tc + k * kout;
+    float b[4];
+    if (VT == 4) {
+      const float4 q = *reinterpret_cast<const float4*>(t);
+      b[0] = q.x; b[1] = q.y; b[2] = q.z; b[3] = q.w;
+    } else if (VT == 2) {
+      const float2 q = *reinterpret_cast<const float2*>(t), p = *reinterpret_cast<const float2*>(t + 2);
+      b[0] = q.x; b[1] = q.y; b[2] = p.x; b[3] = p.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = t[j];
+    }
+    pair_fma(acc[0][0], a0, b[0], b[1]);
+    pair_fma(acc[0][1], a0, b[2], b[3]);
+    pair_fma(acc[1][0], a1, b[0], b[1]);
+    pair_fma(acc[1][1], a1, b[2], b[3]);
+  };
+  for (int k = 0; k < n; k += 4) {
+    const float* x = x0 + (split && k >= map.k0 ? split + k - map.k0 : k);
+    const float4 a0 = *reinterpret_cast<const float4*>(x);
+    const float4 a1 = *reinterpret_cast<const float4*>(x + ldx);
+    step(a0.x, a1.x, k);
+    if (k + 1 < n) step(a0.y, a1.y, k + 1);
+    if (k + 2 < n) step(a0.z, a1.z, k + 2);
+    if (k + 3 < n) step(a0.w, a1.w, k + 3);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int64_t g = row0 + r + i;
+    if (g >= rows) break;
+    float* y = Y + g * ldy + c;
+    const float2 p = acc[i][0], q = acc[i][1];
+    if (vec_y && c + 4 <= kout) {
+      *reinterpret_cast<float4*>(y) = make_float4(p.x, p.y, q.x, q.y);
+    } else {
+      y[0] = p.x;
+      if (c + 1 < kout) y[1] = p.y;
+      if (c + 2 < kout) y[2] = q.x;
+      if (c + 3 < kout) y[3] = q.y;
+    }
+  }
+}
+
 // The same product with T kept in shared memory (n kout up to about 46,000, 200 x 200
 // included): one CTA per SM, each with its own contiguous rows in tiles of wrows 8 RT,
 // so that only X moves during the products and the tiles of a CTA follow each other
@@ -706,6 +793,11 @@ static int vec_cols(const float* X, int ldx, const ColMap& map) {
   return 1;
 }
 
+// whether rows can be copied as they lie (vec: vec_cols), little of them being padding
+static bool straight_rows(int ldx, const ColMap& map, int vec) {
+  return vec == 4 && ldx <= ((map.total() + 7) & ~7) && (map.k1 == 0 || map.ld1 == ldx);
+}
+
 void gram(const float* X, int ldx, ColMap map, int64_t rows, float* G, Workspace& ws,
           cudaStream_t s) {
   const int n = map.total(), ng = (n + kG8 - 1) / kG8;
@@ -723,8 +815,7 @@ void gram(const float* X, int ldx, ColMap map, int64_t rows, float* G, Workspace
   float* partial = ws.gram_partial;
   if (rows > 0) {
     const int vec = vec_cols(X, ldx, map);
-    // straight copies where little of a row is padding
-    const bool straight = vec == 4 && ldx <= ng * kG8 && (map.k1 == 0 || map.ld1 == ldx);
+    const bool straight = straight_rows(ldx, map, vec);
     const int pitch = straight ? ldx : 0;
     const int row = straight ? (map.k1 ? 2 : 1) * ldx : ng * kG8;
     const size_t bytes = (size_t)kGStages * kGRows * row * sizeof(float);
@@ -767,10 +858,27 @@ void gemm_ts(const float* X, int ldx, ColMap map, int64_t rows, const float* T, 
   if (dev < 32 && !(attr.load() & (1u << dev))) {
     for (auto f : {k_gemm_wide<4>, k_gemm_wide<5>, k_gemm_wide<6>, k_gemm_wide<7>, k_gemm_wide<8>})
       SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMWideSmem));
+    for (auto f : {k_gemm_small<1>, k_gemm_small<2>, k_gemm_small<4>})
+      SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMWideSmem));
     const int most = kMStages * (128 * kMLd + kMK * kMaxEll) * (int)sizeof(float);
     for (auto f : {k_gemm_rows<2>, k_gemm_rows<8>})
       SFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
     attr.fetch_or(1u << dev);
+  }
+  // few rows: while their CTAs (up to four an SM, as shared memory allows) take at most
+  // two turns; then T, loaded again for every 16 rows, costs more than the latencies.
+  // us against the other forms, cold: 10,000 x 100 x 100 18 to 24 (two turns), 20,000 x
+  // 100 x 100 26 to 27 (three), 20,000 x 200 x 100 53 to 43 (five).
+  const size_t small_bytes =
+      ((size_t)((n * kout + 7) & ~3) + (size_t)(map.k1 ? 2 : 1) * kSRows * ldx) * sizeof(float);
+  const int64_t small_ctas = (rows + kSRows - 1) / kSRows;
+  if (straight_rows(ldx, map, vec_x) && (uintptr_t)T % 16 == 0 &&
+      small_ctas <= 2 * 152 * (int64_t)std::min<size_t>(4, kMWideSmem / small_bytes)) {
+    const int threads = ((kout + 3) / 4 * (kSRows / 2) + 31) & ~31;
+    auto k = kout % 4 == 0 ? k_gemm_small<4> : kout % 2 == 0 ? k_gemm_small<2> : k_gemm_small<1>;
+    k<<<(unsigned)small_ctas, threads, small_bytes, s>>>(X, ldx, map, rows, T, kout, vec_y, Y, ldy);
+    SFD_LAUNCH_CHECK();
+    return;
   }
   // T in shared memory, one CTA per SM, where the rows fill the SMs (32 or more each; 130
   // against 180 us through the stages at 50,000 x 200 x 200, 24 against 36 at 10,000 x

@@ -48,12 +48,13 @@ def test_gram_is_exact_on_whole_numbers(L, n, pad, offset, rows):
     assert torch.equal(G.double(), Xd.T @ Xd)
 
 
-# 152 x 32 rows is where the resident form begins; 256 x 256 is too large for it
+# rows on both sides of where the forms change: 4864 for 200 columns, 19456 for 100 and
+# fewer; 256 x 256 is too large to stay in shared memory
 @pytest.mark.parametrize("n,kout,padx,pady,offset", [
     (1, 1, 0, 0, 0), (7, 9, 1, 0, 1), (16, 33, 0, 3, 0), (50, 50, 6, 6, 0), (50, 50, 0, 0, 2),
     (100, 100, 4, 4, 0), (100, 97, 0, 1, 3), (129, 65, 3, 7, 0), (200, 200, 0, 0, 0),
     (200, 130, 2, 2, 2), (255, 161, 1, 3, 0), (256, 256, 0, 0, 0)])
-@pytest.mark.parametrize("rows", [1, 63, 4863, 4864, 9731, 40001])
+@pytest.mark.parametrize("rows", [1, 63, 4863, 4864, 4865, 9731, 19456, 19457, 40001])
 def test_product_is_exact_on_whole_numbers(L, n, kout, padx, pady, offset, rows):
     X = block(rows, n, n + padx, offset, n + rows)
     T = block(n, kout, kout, offset, kout)
