@@ -9,7 +9,8 @@
 //   sfd_gemm_ts, 49,999 x 200 x 200                                   418 -> 162
 //   sfd_orthonormalize, 20,000 x 100                                  818 -> 439
 //   sfd_dense_shrink, 200 x 20,000, l = 100                          1494 -> 966
-//   sfd_bssh_buffer, 1,801 x 2,000, l = 50                           2850 -> 2248
+//   sfd_bssh_buffer, 1,801 x 2,000, l = 50                           2850 -> 2248 (2030 with
+//                                                          the few-row X T since)
 #include <string.h>
 
 #include <algorithm>
