@@ -267,7 +267,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512)
     if (k == 0) {
       if (i < n) col = S[i];
     } else {
-      float ks;  // u^T A u
+      float ks;  // u^T p
       if constexpr (NC <= 2) {
         float4 t[4 * NC];
 #pragma unroll
@@ -286,11 +286,11 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512)
         for (int c = 0; c < NC / 2; ++c) ks += kp_s[b][lane + 32 * c];
         ks = warp_sum(ks);
       }
-      const float K = 0.5f * bt * (bt * ks);  // bt^2 alone can overflow
-      const float wk = bt * p_s[b][k] - K * u0;
+      const float K = 0.5f * bt * ks;
+      const float wk = p_s[b][k] - K * u0;
       if (i >= k && i < n) {
         ui = i == k ? u0 : x;
-        wi = bt * p_s[b][i] - K * ui;
+        wi = p_s[b][i] - K * ui;
         col = row_s[b][i] - (ui * wk + wi * u0);
       }
     }
@@ -376,7 +376,9 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512)
         }
       }
     }
-    const float pr = reduce_rows<RW>(acc);
+    // beta joins here, before the next product with u: u^T A u alone is of the size of
+    // the eigenvalue cubed and leaves fp32's range near 1e14 and below 1e-11
+    const float pr = bt * reduce_rows<RW>(acc);
     // lane L holds row W + 16 NC r with r from its top bits
     constexpr int kSh = RW == 8 ? 2 : 3;
     const int re = RW == 8 ? ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)
