@@ -174,6 +174,21 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   return d;
 }
 
+// acc + (a b + c d) on two neighbouring columns: the products are summed first, so that
+// acc, which may be far larger, is rounded once
+__device__ __forceinline__ float2 add_products(float2 acc, float2 a, float2 b, float2 c, float2 d) {
+  float2 r;
+  asm("{\n\t.reg .b64 ra, rb, rc, rd, re;\n\t"
+      "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+      "mov.b64 rd, {%8, %9};\n\tmov.b64 re, {%10, %11};\n\t"
+      "mul.rn.f32x2 rc, rc, rd;\n\tfma.rn.f32x2 ra, ra, rb, rc;\n\t"
+      "add.rn.f32x2 re, re, ra;\n\tmov.b64 {%0, %1}, re;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y), "f"(d.x), "f"(d.y), "f"(acc.x),
+        "f"(acc.y));
+  return r;
+}
+
 // Sum of v[0..RW) over the warp's lanes, each element in the lanes of one group:
 // afterwards lane L holds element elem_of(L) (halving exchanges, so 9 shuffles for 8
 // elements and 8 for 4).
@@ -357,7 +372,9 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(512)
 #pragma unroll
       for (int q = 0; q < QP; ++q) {
         if (64 * q + 63 <= k || 64 * q >= n) continue;
-        A[r][q] = fma2(nw, uq[q], fma2(nu, wq[q], A[r][q]));
+        // (two multiply-adds onto A would round it twice: residuals 1.07 to 1.12 times
+        // these, for 1.5 % of the call at n = 200)
+        A[r][q] = add_products(A[r][q], nw, uq[q], nu, wq[q]);
         a2 = fma2(A[r][q], nq[q], a2);
       }
       acc[r] = a2.x + a2.y;
