@@ -157,10 +157,13 @@ __host__ __device__ constexpr int tri(int I) { return I * (I + 1) / 2; }
 // The shift 2^-20 trace(G) / k keeps the factorisation defined for a rank-deficient
 // block. G is taken times 2^-2e with trace / k in [1, 4) (the result is scaled back
 // by 2^-e, both exact), which keeps pivots and low parts in the normal range.
+template <typename T>
 struct Scale {
-  float sc, shift;  // M = G sc sc + shift I, Rinv = L^-T sc
+  float sc;  // M = G sc sc + shift I, Rinv = L^-T sc
+  T shift;
 };
-__device__ __forceinline__ Scale scale_of(const float* G, int k, float* red /* one per warp */) {
+// red: 2 floats per warp
+__device__ __forceinline__ void scale_of(const float* G, int k, float* red, Scale<float>& S) {
   const int nw = blockDim.x >> 5;
   float tr = 0.f;
   for (int i = threadIdx.x; i < k; i += blockDim.x) tr += G[(int64_t)i * k + i];
@@ -171,8 +174,46 @@ __device__ __forceinline__ Scale scale_of(const float* G, int k, float* red /* o
   tr = 0.f;
   for (int w = 0; w < nw; ++w) tr += red[w];
   const float mean = tr / (float)k;
-  const int e2 = tr > 0.f && isfinite(tr) ? ilogbf(mean) >> 1 : 0;
-  return {ldexpf(1.f, -e2), tr > 0.f ? ldexpf(mean, -20 - 2 * e2) : 1e-30f};
+  const int e2 = mean > 0.f && isfinite(mean) ? ilogbf(mean) >> 1 : 0;
+  S = {ldexpf(1.f, -e2), tr > 0.f ? ldexpf(mean, -20 - 2 * e2) : 1e-30f};
+}
+// The trace of the accurate form is a two-float sum of the diagonal times 2^-e, with e
+// the exponent of its largest entry: a trace may exceed the largest float where no entry
+// of G does.
+__device__ __forceinline__ void scale_of(const float* G, int k, float* red, Scale<DF>& S) {
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float big = 0.f;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) big = fmaxf(big, fabsf(G[(int64_t)i * k + i]));
+  const unsigned bits = __reduce_max_sync(kFull, __float_as_uint(big));
+  if (lane == 0) red[warp] = __uint_as_float(bits);
+  __syncthreads();
+  for (int w = 0; w < nw; ++w) big = fmaxf(big, red[w]);
+  const int e = big > 0.f && isfinite(big) ? ilogbf(big) : 0;
+  __syncthreads();
+  auto add = [](DF a, DF b) {
+    const DF s = df_two_sum(a.h, b.h);
+    return df_fast(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+  };
+  DF tr = {0.f, 0.f};
+  for (int i = threadIdx.x; i < k; i += blockDim.x)
+    tr = add(tr, {ldexpf(G[(int64_t)i * k + i], -e), 0.f});
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    tr = add(tr, {__shfl_xor_sync(kFull, tr.h, o), __shfl_xor_sync(kFull, tr.l, o)});
+  if (lane == 0) {
+    red[2 * warp] = tr.h;
+    red[2 * warp + 1] = tr.l;
+  }
+  __syncthreads();
+  tr = {0.f, 0.f};
+  for (int w = 0; w < nw; ++w) tr = add(tr, {red[2 * w], red[2 * w + 1]});
+  const float kf = (float)k, q = __fdiv_rn(tr.h, kf);
+  const DF mean = df_fast(q, __fdiv_rn(__fadd_rn(__fmaf_rn(-q, kf, tr.h), tr.l), kf));
+  const bool pos = tr.h > 0.f;
+  const int e2 = pos && isfinite(tr.h) ? (ilogbf(mean.h) + e) >> 1 : 0;
+  const int es = e - 20 - 2 * e2;
+  S.sc = ldexpf(1.f, -e2);
+  S.shift = pos ? DF{ldexpf(mean.h, es), ldexpf(mean.l, es)} : DF{1e-30f, 0.f};
 }
 
 // CW chain warps (a lane per column), NTW tile warps with TPT tiles per thread.
@@ -183,7 +224,7 @@ __global__ void __launch_bounds__(32 * (CW + NTW))
   constexpr int kLd = 32 * CW;  // columns of X and W
   constexpr int kPl = kTwo<T> ? 2 : 1;
   __shared__ __align__(16) float xw[4][kPl][4 * kLd];  // X and W of the even and odd pivots
-  __shared__ float red[CW + NTW];
+  __shared__ float red[2 * (CW + NTW)];
   const int NB = (k + 3) >> 2;
   const int tid = threadIdx.x, warp = tid >> 5;
   auto rows = [&](int i) {
@@ -216,9 +257,11 @@ __global__ void __launch_bounds__(32 * (CW + NTW))
         m[n][r][q] = c_val<T>(I[n] < 0 ? 0.f : a < k ? G[(int64_t)a * k + b] : i == j ? 1.f : 0.f);
       }
   }
-  const Scale S = scale_of(G, k, red);
+  Scale<T> S;
+  scale_of(G, k, red, S);
   const float sc = S.sc;
-  const T shift = c_val<T>(S.shift);
+  const T shift = S.shift;
+  const float least = c_out(shift);  // in place of a pivot that is not positive
   // tiles of pivot P's row and column into X
   auto publish = [&](int n, int P) {
     const Rows<T> X = rows(P & 1);
@@ -292,7 +335,7 @@ __global__ void __launch_bounds__(32 * (CW + NTW))
       for (int j = 0; j < 4; ++j) {
         const bool pos = c_pos(d[j][j]);
         clamped += !pos;
-        inv[j] = c_rsqrt(pos ? d[j][j] : shift);
+        inv[j] = c_rsqrt(pos ? d[j][j] : c_val<T>(least));
 #pragma unroll
         for (int r = j + 1; r < 4; ++r) d[r][j] = c_mul(d[r][j], inv[j]);
 #pragma unroll
@@ -383,7 +426,7 @@ __host__ __device__ constexpr int r_ld(int KP) { return KP + 4; }
 // current one's reciprocal root is known, so a column costs one root and two
 // multiply-adds in sequence, and the shuffles of the updates overlap the next root.
 template <typename T>
-__device__ __forceinline__ void diag_block(Rows<T> M, Rows<T> R, int ldr, Rows<T> Li, int I, T shift,
+__device__ __forceinline__ void diag_block(Rows<T> M, Rows<T> R, int ldr, Rows<T> Li, int I, float least,
                                            int& clamped) {
   const int lane = threadIdx.x & 31, i = lane & 15, h = lane >> 4;
   T d[8], x[8];
@@ -419,7 +462,7 @@ __device__ __forceinline__ void diag_block(Rows<T> M, Rows<T> R, int ldr, Rows<T
       const T q = c_shfl(d[sub], ((j + 1) & 15) | (own ^ 16));
       const bool pos = c_pos(piv);
       clamped += !pos;
-      const T inv = c_rsqrt(pos ? piv : shift);
+      const T inv = c_rsqrt(pos ? piv : c_val<T>(least));
       const T l = i > j ? c_mul(dj, inv) : c_val<T>(0.f);
       const T nl = c_neg(l), ln = c_mul(c, inv);
       piv = q;
@@ -549,11 +592,13 @@ __global__ void __launch_bounds__(kPanelThreads)
     Li.q = R.q + rsz;
     M.q = kLoGlobal ? lo_work : Li.q + kCB * kLiLd;
   }
-  __shared__ float red[16];
+  __shared__ float red[2 * (kPanelThreads / 32)];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
 
-  const Scale S = scale_of(G, k, red);
-  const T shift = c_val<T>(S.shift);
+  Scale<T> S;
+  scale_of(G, k, red, S);
+  const T shift = S.shift;
+  const float least = c_out(shift);  // in place of a pivot that is not positive
   // the lower triangle of G, a warp per row; padding rows are the identity
   for (int i = warp; i < KP; i += nw) {
     const int I = i >> 4, o = m_off(I) + (i & 15) * m_ld(I), w = kCB * (I + 1);
@@ -570,7 +615,7 @@ __global__ void __launch_bounds__(kPanelThreads)
   for (int p = 0; p <= NB; ++p) {
     // ---- c for panel p - 1 (block row I has (I + 2) / 2 tiles), a for panel p
     if (warp == 0) {
-      if (p < NB) diag_block<T>(M, R, ldr, Li, p, shift, clamped);
+      if (p < NB) diag_block<T>(M, R, ldr, Li, p, least, clamped);
     } else if (p > 0) {
       int I = p, nt = (p + 1) / 2, rem = warp - 1;  // row p without its diagonal block
       for (;;) {
