@@ -249,7 +249,7 @@ int sfd_dense_shrink(int64_t rows, int64_t d, int32_t ell, const float* M, float
       d > 2000000)
     return SFD_EINVAL;
   return guarded([&]() -> int {
-    ScratchLease L(true);
+    ScratchLease L;
     Merger G(d, ell, L.s);
     // rows 0..min(rows,l) are the "B" block, the rest the stacked block
     const int k0 = (int)std::min<int64_t>(rows, ell);
