@@ -201,8 +201,9 @@ const char* sfd_last_error(const sfd_ctx* ctx);
 /* ------------------------------------------------------------------------
  * One buffer / one stack (the per-step calls used to check each stage).
  * Device pointers only; the stream is the default stream of the calling
- * thread's current device. Scratch is kept between calls (512 MB at most) and
- * freed by sfd_destroy, sfd_batch_destroy and when an allocation fails.
+ * thread's current device. Scratch is kept between calls (512 MB at most per
+ * CUDA context) and freed by sfd_destroy, sfd_batch_destroy and when an
+ * allocation fails, each for the calling thread's current CUDA context.
  * ------------------------------------------------------------------------ */
 
 /* BoostedSparseShrink (Alg. 4) of one buffer A' (m x d CSR with int32

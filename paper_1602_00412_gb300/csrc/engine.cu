@@ -57,10 +57,42 @@ void alloc_sort(DevArena& A, SortBuffers& t, Workspace& ws, int64_t nnz, int64_t
 
 namespace {
 
-// idle scratches, the most recent last; guarded by g_scratch_m
+// idle scratches of every context, the most recent first; guarded by g_scratch_m
 std::mutex g_scratch_m;
-Scratch* g_scratch_idle[kScratchIdle];
-int g_scratch_count = 0;
+Scratch* g_scratch_idle = nullptr;
+
+// to the idle ones of its context, or freed when these are enough (its stream is idle)
+void give_back(Scratch* s) {
+  bool keep = s->ctx_id != 0;
+  if (keep) {
+    std::lock_guard<std::mutex> lock(g_scratch_m);
+    size_t held = s->bytes;
+    int count = 0;
+    for (Scratch* c = g_scratch_idle; c; c = c->next)
+      if (c->ctx_id == s->ctx_id) {
+        held += c->bytes;
+        ++count;
+      }
+    keep = count < kScratchIdle && held <= kScratchKeep;
+    if (keep) {
+      s->next = g_scratch_idle;
+      g_scratch_idle = s;
+    }
+  }
+  if (!keep) delete s;
+}
+
+// the most recent idle one of context id, or null
+Scratch* take(unsigned long long id) {
+  std::lock_guard<std::mutex> lock(g_scratch_m);
+  for (Scratch** at = &g_scratch_idle; *at; at = &(*at)->next)
+    if ((*at)->ctx_id == id) {
+      Scratch* s = *at;
+      *at = s->next;
+      return s;
+    }
+  return nullptr;
+}
 
 }  // namespace
 
@@ -76,7 +108,6 @@ cudaError_t device_malloc(void** p, size_t bytes) {
 
 Scratch::Scratch() {
   try {
-    SFD_CUDA(cudaGetDevice(&dev));
     SFD_CUDA(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
     SFD_CUDA(cudaEventCreateWithFlags(&event, cudaEventDisableTiming));
     void* p = nullptr;
@@ -117,73 +148,44 @@ char* Scratch::reserve(size_t n) {
 }
 
 ScratchLease::ScratchLease(bool all_streams) : s(nullptr) {
-  int dev = 0;
   unsigned long long id = 0;
-  SFD_CUDA(cudaGetDevice(&dev));
   SFD_CUDA(cudaFree(nullptr));  // the context exists from here on
   if (!current_ctx_id(&id)) id = 0;
-  {
-    std::lock_guard<std::mutex> lock(g_scratch_m);
-    for (int i = g_scratch_count; i-- > 0 && !s;) {
-      Scratch* c = g_scratch_idle[i];
-      if (c->dev != dev) continue;
-      for (int j = i + 1; j < g_scratch_count; ++j) g_scratch_idle[j - 1] = g_scratch_idle[j];
-      --g_scratch_count;
-      if (c->ctx_id == id) s = c;
-      else ::operator delete(c);  // of a context that is gone, and its memory with it
-    }
+  if (all_streams) {
+    SFD_CUDA(cudaDeviceSynchronize());
+  } else {
+    // An allocation is what CUDA refuses while a capture is under way whose work has
+    // not run yet (the input may be its output), so the call is refused then, also
+    // when its memory is there already; a small one takes 2 us.
+    void* probe = nullptr;
+    SFD_CUDA(cudaMalloc(&probe, 256));
+    SFD_CUDA(cudaFree(probe));
   }
+  if (id) s = take(id);
   if (!s) s = new Scratch();
-  try {
-    if (all_streams) {
-      SFD_CUDA(cudaDeviceSynchronize());
-    } else {
-      // An allocation is what CUDA refuses while a capture is under way whose work has
-      // not run yet (the input may be its output), so the call is refused then, also
-      // when its memory is there already; a small one takes 2 us.
-      void* probe = nullptr;
-      SFD_CUDA(cudaMalloc(&probe, 256));
-      SFD_CUDA(cudaFree(probe));
-      SFD_CUDA(cudaEventRecord(s->event, 0));
-      SFD_CUDA(cudaStreamWaitEvent(s->stream, s->event, 0));
-    }
-  } catch (...) {
-    delete s;
-    throw;
+  if (all_streams) return;
+  cudaError_t e = cudaEventRecord(s->event, 0);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(s->stream, s->event, 0);
+  if (e != cudaSuccess) {
+    give_back(s);
+    throw CudaError{e, "order after the caller's stream"};
   }
 }
 
 ScratchLease::~ScratchLease() {
-  bool keep = cudaStreamSynchronize(s->stream) == cudaSuccess && s->ctx_id != 0;
-  if (keep) {
-    std::lock_guard<std::mutex> lock(g_scratch_m);
-    size_t held = s->bytes;
-    for (int i = 0; i < g_scratch_count; ++i) held += g_scratch_idle[i]->bytes;
-    keep = g_scratch_count < kScratchIdle && held <= kScratchKeep;
-    if (keep) g_scratch_idle[g_scratch_count++] = s;
-  }
-  if (!keep) delete s;
+  if (cudaStreamSynchronize(s->stream) == cudaSuccess) give_back(s);
+  else delete s;
 }
 
 void scratch_trim() {
-  Scratch* idle[kScratchIdle];
-  int n;
   {
     std::lock_guard<std::mutex> lock(g_scratch_m);
-    n = g_scratch_count;
-    std::copy(g_scratch_idle, g_scratch_idle + n, idle);
-    g_scratch_count = 0;
+    if (!g_scratch_idle) return;
   }
-  if (n == 0) return;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  for (int i = 0; i < n; ++i) {
-    unsigned long long id = 0;
-    cudaSetDevice(idle[i]->dev);
-    if (current_ctx_id(&id) && id == idle[i]->ctx_id) delete idle[i];
-    else ::operator delete(idle[i]);
-  }
-  cudaSetDevice(dev);
+  // not while frees are refused (a capture), nor in another context than theirs
+  unsigned long long id = 0;
+  if (cudaFree(nullptr) != cudaSuccess || !current_ctx_id(&id) || id == 0) return;
+  while (Scratch* s = take(id)) delete s;
 }
 
 void clear_dense_scratch(Workspace& ws, cudaStream_t s) {

@@ -26,16 +26,18 @@ namespace sfd {
 // and an event. Creating and freeing these cost several times the kernels of most
 // calls (a Gram of 50,000 x 100: 274 us a call, 20 us of kernels; 43 us a call now), so a finished call
 // leaves them to the next one. A call holds its Scratch alone, whatever its thread or
-// stream. At most kScratchIdle idle ones of kScratchKeep bytes together are kept, each
-// for its own CUDA context; they are freed when an allocation of the library fails and
-// when a context (sfd_destroy) or a batch is destroyed.
+// stream. Of each CUDA context at most kScratchIdle idle ones of kScratchKeep bytes
+// together are kept; they are used and freed with that context current and not touched
+// otherwise (a context that ends takes its memory along and leaves the small host
+// structs; ids of contexts are never reused). They are freed when an allocation of the
+// library fails and when a context (sfd_destroy) or a batch is destroyed.
 constexpr int kScratchIdle = 4;
 constexpr size_t kScratchKeep = (size_t)512 << 20;
 constexpr size_t kScratchPinned = 4096;
 
 struct Scratch {
-  int dev = 0;
-  unsigned long long ctx_id = 0;
+  unsigned long long ctx_id = 0;  // 0: unknown, not kept
+  Scratch* next = nullptr;        // of the idle list
   cudaStream_t stream = nullptr;
   cudaEvent_t event = nullptr;
   char* block = nullptr;
@@ -60,7 +62,7 @@ struct ScratchLease {
   ScratchLease& operator=(const ScratchLease&) = delete;
   Scratch* operator->() { return s; }
 };
-void scratch_trim();  // free the idle ones of every thread
+void scratch_trim();  // free the current context's idle ones, whatever thread used them
 // cudaMalloc; on failure once more after scratch_trim
 cudaError_t device_malloc(void** p, size_t bytes);
 // Id of the calling thread's current CUDA context (0 when there is none).
