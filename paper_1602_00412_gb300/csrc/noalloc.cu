@@ -55,27 +55,31 @@ using CtxGetId = CUresult (*)(CUcontext, unsigned long long*);
 
 }  // namespace
 
-// Id of the calling thread's current context (0 when there is none).
+// Id of the calling thread's current context (0 when there is none). Called by several
+// threads at once: the entry points are looked up once, behind a static's guard.
 bool current_ctx_id(unsigned long long* id) {
-  static CtxGetCurrent get_current = nullptr;
-  static CtxGetId get_id = nullptr;
-  if (!get_current || !get_id) {
-    void* a = nullptr;
-    void* b = nullptr;
-    cudaDriverEntryPointQueryResult qa, qb;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa) !=
-            cudaSuccess ||
-        cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb) !=
-            cudaSuccess ||
-        qa != cudaDriverEntryPointSuccess || qb != cudaDriverEntryPointSuccess || !a || !b)
-      return false;
-    get_current = reinterpret_cast<CtxGetCurrent>(a);
-    get_id = reinterpret_cast<CtxGetId>(b);
-  }
+  struct Entry {
+    CtxGetCurrent get_current = nullptr;
+    CtxGetId get_id = nullptr;
+    Entry() {
+      void* a = nullptr;
+      void* b = nullptr;
+      cudaDriverEntryPointQueryResult qa, qb;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa) !=
+              cudaSuccess ||
+          cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb) !=
+              cudaSuccess ||
+          qa != cudaDriverEntryPointSuccess || qb != cudaDriverEntryPointSuccess)
+        return;
+      get_current = reinterpret_cast<CtxGetCurrent>(a);
+      get_id = reinterpret_cast<CtxGetId>(b);
+    }
+  };
+  static const Entry e;
   CUcontext ctx = nullptr;
-  if (get_current(&ctx) != CUDA_SUCCESS) return false;
+  if (!e.get_current || !e.get_id || e.get_current(&ctx) != CUDA_SUCCESS) return false;
   *id = 0;
-  return !ctx || get_id(ctx, id) == CUDA_SUCCESS;
+  return !ctx || e.get_id(ctx, id) == CUDA_SUCCESS;
 }
 
 namespace {
