@@ -189,7 +189,9 @@ int sfd_get_stats(const sfd_ctx* ctx, sfd_stats* out);
  * cleared. Device memory is kept. */
 int sfd_reset(sfd_ctx* ctx);
 
-/* Release every resource of the context (NULL is a no-op). */
+/* Release every resource of the context (NULL: of no context), and the scratch
+ * that stage calls left: a program of stage calls alone gives it back by
+ * sfd_destroy(NULL). */
 void sfd_destroy(sfd_ctx* ctx);
 
 /* Static text for a status code. */

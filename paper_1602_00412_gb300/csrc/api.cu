@@ -330,7 +330,7 @@ int sfd_create(int64_t d, int32_t ell, uint64_t seed, const sfd_options* opt, sf
 
 void sfd_destroy(sfd_ctx* ctx) {
   delete ctx;
-  if (ctx) scratch_trim();
+  scratch_trim();
 }
 
 int sfd_append_rows(sfd_ctx* ctx, int64_t nrows, const int64_t* indptr, const int32_t* indices,

@@ -164,3 +164,26 @@ def test_stages_repeat_their_bits(sfd):
         p.check(sfd.load())
     for again in (run(), run()):
         assert all(torch.equal(a, b) for a, b in zip(first, again))
+
+
+def test_scratch_given_back_without_a_sketch(sfd):
+    # a program of stage calls alone: sfd_destroy(NULL) frees what they left
+    L = sfd.load()
+    rows, k = 400000, 64
+    X = torch.ones((rows, k), device="cuda")
+    G = torch.empty((k, k), device="cuda")
+
+    def call():
+        assert L.sfd_orthonormalize(rows, k, ptr(X), k) == 0  # 100 MB of scratch
+        assert L.sfd_gram(rows, k, ptr(X), k, ptr(G), 0) == 0
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    call()
+    L.sfd_destroy(None)
+    free = torch.cuda.mem_get_info()[0]
+    assert free - call() >= 100 << 20
+    L.sfd_destroy(None)
+    assert torch.cuda.mem_get_info()[0] == free
+    L.sfd_destroy(None)
+    call()
