@@ -212,7 +212,10 @@ const char* sfd_last_error(const sfd_ctx* ctx);
  * rowptr[m+1] starting at 0, colidx[nnz], vals[nnz], device memory), with the
  * randomness of buffer index b under `seed` (same keys as a context).
  * l <= m is required (Alg. 3). Output Bp_out: l x d row-major (device), the
- * shrunk sketch B' = Lambda~ V^T. info may be NULL. opt may be NULL. */
+ * shrunk sketch B' = Lambda~ V^T. info may be NULL. opt may be NULL; of it this
+ * call reads delta, verify, c_q, q_override, retry_cap and inject_vs_fail only:
+ * it runs in FP32 with the fixed schedule whatever precision and q_mode say
+ * (those are a context's). */
 int sfd_bssh_buffer(int64_t m, int64_t d, int32_t ell, const int32_t* rowptr, const int32_t* colidx,
                     const float* vals, uint64_t seed, int64_t b, const sfd_options* opt,
                     float* Bp_out, sfd_shrink_info* info);

@@ -237,6 +237,7 @@ def sfd_load(blob, runtime=None):
 
 
 def sfd_bssh_buffer(m, d, ell, rowptr, colidx, vals, seed, b, Bp_out, opts=None):
+    """One buffer's BoostedSparseShrink, in FP32 whatever opts.precision says."""
     info = sfd_shrink_info()
     _check(load().sfd_bssh_buffer(m, d, ell, ctypes.c_void_p(rowptr.data_ptr()),
                                   ctypes.c_void_p(colidx.data_ptr()),

@@ -189,3 +189,15 @@ def test_dense_shrink_matches_oracle(lib, rows, d, ell):
     # fp32 Gram + eigensolve of an n x n problem (n = rows): relative error ~ n u
     tol = max(1e-5, 2 * rows * 2.0 ** -24)
     assert bbt_rel_diff(got, ref) < tol
+
+
+def test_bssh_buffer_is_fp32_whatever_precision_says(lib):
+    # precision is an option of contexts; the stage call is documented to run in FP32
+    X = synth.planted(600, 500, 20, 1.1, 5, 10.0, 0.7, 0.1, 4)
+    out = []
+    for precision in (0, 1):
+        Bp = torch.zeros((50, 500), device="cuda")
+        lib.sfd_bssh_buffer(500, 500, 50, dev(X.indptr[:501], np.int32), dev(X.indices),
+                            dev(X.values), 7, 0, Bp, lib.options(precision=precision))
+        out.append(Bp.cpu())
+    assert float(out[0].norm()) > 0 and torch.equal(out[0], out[1])
