@@ -298,28 +298,23 @@ __global__ void __launch_bounds__(512)
   G[(int64_t)c * n + a] = t;
 }
 
-// G[e] = sum over chunks of the partial tiles. A block takes 32 consecutive
-// output elements; its 8 warps each sum every 8th chunk (coalesced 128-byte
-// reads per chunk), and the 8 warp sums are added in a fixed order, so the
-// result does not depend on scheduling.
+// G[e] = sum over chunks of the tensor-core Grams' partial tiles (one 128 x 128 tile
+// each). A block takes 32 consecutive output elements; its 8 warps each sum every 8th
+// chunk (coalesced 128-byte reads per chunk), and the 8 warp sums are added in a fixed
+// order, so the result does not depend on scheduling.
 constexpr int kRedGroups = 8;
 
 __global__ void __launch_bounds__(32 * kRedGroups)
-    k_gram_reduce(const float* __restrict__ partial, int nchunks, int npairs, int ntiles, int n,
-                  float* __restrict__ G) {
+    k_gram_reduce(const float* __restrict__ partial, int nchunks, int n, float* __restrict__ G) {
   __shared__ float sums[kRedGroups][33];
   const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   const int64_t e = (int64_t)blockIdx.x * 32 + lane;
   const bool live = e < (int64_t)n * n;
   float acc = 0.f;
   if (live) {
-    int a = (int)(e / n), c = (int)(e % n);
-    if (a / kT > c / kT) { int t = a; a = c; c = t; }   // use the upper tile (ti <= tj)
-    const int ti = a / kT, tj = c / kT;
-    const int tp = ti * ntiles - ti * (ti - 1) / 2 + (tj - ti);
-    const int off = (a % kT) * kT + (c % kT);
-    const float* p = partial + (int64_t)tp * (kT * kT) + off;
-    const int64_t stride = (int64_t)npairs * (kT * kT);
+    const int a = (int)(e / n), c = (int)(e % n);
+    const float* p = partial + a * kT + c;
+    constexpr int64_t stride = kT * kT;
     // chunks grp, grp + 16, ... into s0 and grp + 8, grp + 24, ... into s1,
     // in that order; eight loads are issued before their adds
     float s0 = 0.f, s1 = 0.f;
@@ -435,22 +430,23 @@ __device__ __forceinline__ void async_t_row(float* dst, const float* T, int kk, 
 }
 
 template <int RT>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(256)
     k_gemm_rows(const float* __restrict__ X, int ldx, ColMap map, int64_t rows,
-                const float* __restrict__ T, int kout, int wrows, int wcols, int vec_x, int vec_t,
+                const float* __restrict__ T, int kout, int wcols, int vec_x, int vec_t,
                 bool vec_y, float* __restrict__ Y, int ldy) {
   extern __shared__ __align__(16) float sm[];
   const int n = map.total();
   const int ps = wcols * 16, ts = 2 * ps;  // T stage: half and whole row, in floats
-  const int xfl = wrows * 8 * RT * kMLd, stage = xfl + kMK * ts;
+  constexpr int xfl = 8 * RT * kMLd;
+  const int stage = xfl + kMK * ts;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int r_lane = (warp / wcols) * 8 * RT + (lane >> 2), tc = (warp % wcols) * 4 + (lane & 3);
-  const int64_t row0 = (int64_t)blockIdx.x * wrows * 8 * RT;
+  const int r_lane = lane >> 2, tc = warp * 4 + (lane & 3);  // a warp per 32 columns
+  const int64_t row0 = (int64_t)blockIdx.x * 8 * RT;
   const int nst = (n + kMK - 1) / kMK;
   auto load = [&](int st) {
     float* xs = sm + (st % kMStages) * stage;
     float* tb = xs + xfl;
-    for (int i = tid; i < wrows * 8 * RT * (kMK / 4); i += blockDim.x) {
+    for (int i = tid; i < 8 * RT * (kMK / 4); i += blockDim.x) {
       const int r = i >> 2, q = i & 3;
       const int64_t g = row0 + r;
       async_cols(xs + r * kMLd + 4 * q, X, ldx, map, g, st * (kMK / 4) + q, g < rows, vec_x);
@@ -839,7 +835,7 @@ void gram(const float* X, int ldx, ColMap map, int64_t rows, float* G, Workspace
 
 void gram_reduce_tiles(const float* partial, int nchunks, int n, float* G, cudaStream_t s) {
   int64_t ne = (int64_t)n * n;
-  k_gram_reduce<<<(unsigned)((ne + 31) / 32), 32 * kRedGroups, 0, s>>>(partial, nchunks, 1, 1, n, G);
+  k_gram_reduce<<<(unsigned)((ne + 31) / 32), 32 * kRedGroups, 0, s>>>(partial, nchunks, n, G);
   SFD_LAUNCH_CHECK();
 }
 
@@ -911,15 +907,16 @@ void gemm_ts(const float* X, int ldx, ColMap map, int64_t rows, const float* T, 
   const size_t bytes = (size_t)kMStages * (tile * kMLd + kMK * wcols * 32) * sizeof(float);
   auto k = rt == 2 ? k_gemm_rows<2> : k_gemm_rows<8>;
   k<<<(unsigned)((rows + tile - 1) / tile), wcols * 32, bytes, s>>>(
-      X, ldx, map, rows, T, kout, 1, wcols, vec_x, vec_t, vec_y, Y, ldy);
+      X, ldx, map, rows, T, kout, wcols, vec_x, vec_t, vec_y, Y, ldy);
   SFD_LAUNCH_CHECK();
 }
 
 void chol_inv(const float* G, int k, float* Rinv, float* work, int* flags, cudaStream_t s,
               bool accurate) {
-  // the blocked in-place form holds its triangle in one SM's shared memory up to
-  // k = 256 (every block the method orthonormalises); only eigenvector blocks
-  // (fp32) are wider, and go a column at a time through global memory
+  // the in-place forms serve k <= 256 (every block the method orthonormalises): the
+  // triangle in registers, above that in shared memory, its low parts in global memory
+  // where both do not fit (two-float, k > 208); only eigenvector blocks (fp32) are
+  // wider, and go a column at a time through global memory
   if (k <= kMaxEll) {
     chol_inv_blk(G, k, Rinv, work, flags, s, accurate);
     return;
