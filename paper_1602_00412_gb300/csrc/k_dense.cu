@@ -79,9 +79,11 @@ __global__ void k_gauss_fill(float* __restrict__ out, int64_t rows, int cols, in
 // stages, as a straight copy where rows are contiguous (k_gram_tri). The multiply-adds
 // are packed two columns at a time (half the issue slots; each is rounded as fmaf) and
 // bound the kernel: 64 per thread and row against 4 shared float4 loads.
-// Cold, with its reduction: 100,000 x 200 128 us (31 TFLOP/s counting both triangles; 438
+// Cold, with its reduction: 100,000 x 200 128 us (31 TFLOP/s, one triangle counted; 438
 // in 128 x 128 tiles, 168 with row by row copies), 20,000 x 100 23 us (49, 25), 2,000 x
-// 50 11 us (15 with row by row copies).
+// 50 11 us (15 with row by row copies). Rows of any other alignment go row by row, their
+// copies spread over all threads: 200,000 x 33 at a pitch of 33 107 us (200 in 128 x 128
+// tiles, 267 with a warp per row), 400,000 x 1 104 (333, 435).
 constexpr int kT = 128;  // output tile of the tensor-core Grams' partials
 constexpr int kG8 = 8;
 constexpr int kGRows = 16;    // rows per stage
@@ -147,6 +149,21 @@ __device__ __forceinline__ void async_cols(float* dst, const float* X, int ldx, 
   }
 }
 
+// The indices i, i + step, .. as (row r, column c) of rows of w, without a division each.
+struct Grid2 {
+  int r, c, dr, dc, w;
+  __device__ __forceinline__ Grid2(int i, int step, int width)
+      : r(i / width), c(i % width), dr(step / width), dc(step % width), w(width) {}
+  __device__ __forceinline__ void next() {
+    r += dr;
+    c += dc;
+    if (c >= w) {
+      c -= w;
+      ++r;
+    }
+  }
+};
+
 // partial[chunk][tile][64]: tiles of the upper triangle in row-major order.
 // pitch: floats between rows, of both blocks, when a stage is 16 pitch floats of each
 // block as they lie (both start on 16 bytes, pitch and the first block's width are
@@ -160,7 +177,7 @@ __global__ void __launch_bounds__(512)
   const int rs = pitch ? pitch : ng * kG8;  // floats between rows of a stage
   const int split = pitch && map.k1 ? kGRows * rs : 0;  // where its second block begins
   const int stage = split ? 2 * split : kGRows * rs;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x;
   const int slot = (int)(blockIdx.y * blockDim.x) + tid, e = min(slot, ntiles - 1);
   int ti = 0, start = 0;
   {  // row ti of the triangle starts at ti ng - ti (ti - 1) / 2
@@ -200,9 +217,9 @@ __global__ void __launch_bounds__(512)
         }
       }
     } else {
-      for (int r = warp; r < kGRows; r += nw)
-        for (int c4 = lane; c4 < 2 * ng; c4 += 32)
-          async_cols(buf + r * rs + 4 * c4, X, ldx, map, r0 + r, c4, r0 + r < r_end, vec);
+      Grid2 at(tid, blockDim.x, 2 * ng);  // c: group of four columns
+      for (; at.r < kGRows; at.next())
+        async_cols(buf + at.r * rs + 4 * at.c, X, ldx, map, r0 + at.r, at.c, r0 + at.r < r_end, vec);
     }
   };
   float2 acc[8][4];
