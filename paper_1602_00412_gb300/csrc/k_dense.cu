@@ -428,20 +428,30 @@ __device__ __forceinline__ void gemm_store(const float2 (&acc)[RT][4], float* Y,
   }
 }
 
-// row kk of T (zero past n rows and kout columns) by one warp, in copies of vec_t columns
-__device__ __forceinline__ void async_t_row(float* dst, const float* T, int kk, int n, int kout,
-                                            int wcols, int vec_t) {
-  const int ps = wcols * 16;
-  for (int c4 = threadIdx.x & 31; c4 < wcols * 8; c4 += 32) {
-    float* d = dst + (c4 & 1) * ps + (c4 >> 1) * 4;
+// rows k0 .. k0 + count - 1 of T (zero past n rows and kout columns), ts floats apart at
+// dst, by all threads in copies of vec_t columns
+__device__ __forceinline__ void async_t_rows(float* dst, const float* T, int k0, int count, int n,
+                                             int kout, int wcols, int vec_t) {
+  const int ps = wcols * 16, ts = 2 * ps;
+  if (vec_t == 1) {  // neighbouring threads take neighbouring columns
+    for (Grid2 at(threadIdx.x, blockDim.x, wcols * 32); at.r < count; at.next()) {
+      const int kk = k0 + at.r, c = at.c;
+      const bool ok = kk < n && c < kout;
+      async_copy4(dst + at.r * ts + ((c >> 2) & 1) * ps + (c >> 3) * 4 + (c & 3),
+                  ok ? T + (int64_t)kk * kout + c : T, ok);
+    }
+    return;
+  }
+  for (Grid2 at(threadIdx.x, blockDim.x, wcols * 8); at.r < count; at.next()) {
+    const int kk = k0 + at.r, c4 = at.c;
+    float* d = dst + at.r * ts + (c4 & 1) * ps + (c4 >> 1) * 4;
     const float* src = T + (int64_t)kk * kout + 4 * c4;
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
+    for (int t = 0; t < 4; t += 2) {
       if (t % vec_t) continue;
       const bool ok = kk < n && 4 * c4 + t < kout;
       if (vec_t == 4) async_copy16(d, ok ? src : T, ok ? 16 : 0);
-      else if (vec_t == 2) async_copy8(d + t, ok ? src + t : T, ok ? 8 : 0);
-      else async_copy4(d + t, ok ? src + t : T, ok);
+      else async_copy8(d + t, ok ? src + t : T, ok ? 8 : 0);
     }
   }
 }
@@ -456,7 +466,7 @@ __global__ void __launch_bounds__(256)
   const int ps = wcols * 16, ts = 2 * ps;  // T stage: half and whole row, in floats
   constexpr int xfl = 8 * RT * kMLd;
   const int stage = xfl + kMK * ts;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r_lane = lane >> 2, tc = warp * 4 + (lane & 3);  // a warp per 32 columns
   const int64_t row0 = (int64_t)blockIdx.x * 8 * RT;
   const int nst = (n + kMK - 1) / kMK;
@@ -468,8 +478,7 @@ __global__ void __launch_bounds__(256)
       const int64_t g = row0 + r;
       async_cols(xs + r * kMLd + 4 * q, X, ldx, map, g, st * (kMK / 4) + q, g < rows, vec_x);
     }
-    for (int k = warp; k < kMK; k += nw)
-      async_t_row(tb + k * ts, T, st * kMK + k, n, kout, wcols, vec_t);
+    async_t_rows(tb, T, st * kMK, kMK, n, kout, wcols, vec_t);
   };
   float2 acc[RT][4];
 #pragma unroll
@@ -595,7 +604,7 @@ __global__ void __launch_bounds__(512)
   const int ps = wcols * 16, ts = 2 * ps;
   const int nst = (n + kMK - 1) / kMK, tile = wrows * 8 * RT, xfl = tile * kMLd;
   float* xbuf = sm + nst * kMK * ts;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r_lane = (warp / wcols) * 8 * RT + (lane >> 2), tc = (warp % wcols) * 4 + (lane & 3);
   const int64_t r_beg = (int64_t)blockIdx.x * rows_per_cta;
   const int64_t r_end = min(rows, r_beg + rows_per_cta);
@@ -609,7 +618,7 @@ __global__ void __launch_bounds__(512)
                  row0 + r < r_end, vec_x);
     }
   };
-  for (int k = warp; k < nst * kMK; k += nw) async_t_row(sm + k * ts, T, k, n, kout, wcols, vec_t);
+  async_t_rows(sm, T, 0, nst * kMK, n, kout, wcols, vec_t);
   float2 acc[RT][4];
 #pragma unroll
   for (int i = 0; i < RT; ++i)
@@ -895,32 +904,40 @@ void gemm_ts(const float* X, int ldx, ColMap map, int64_t rows, const float* T, 
   }
   // T in shared memory, one CTA per SM, where the rows fill the SMs (32 or more each; 130
   // against 180 us through the stages at 50,000 x 200 x 200, 24 against 36 at 10,000 x
-  // 100 x 100), with the rows per thread that waste least of the last tile
+  // 100 x 100), with the rows of warps and the rows per thread that waste least of the
+  // last tile: narrow outputs, whose 16 warps would cover 512 rows and more, take fewer
+  // (20,011 x 200 x 20: 30 us, 79 with 16; 10,000 x 50 x 3: 9 and 26)
   const size_t t_bytes = (size_t)((n + kMK - 1) / kMK) * kMK * wcols * 32 * sizeof(float);
-  const int wide_rows = std::max(1, 16 / wcols);
+  const int most_rows = std::max(1, 16 / wcols);
   const size_t x_row = (size_t)kMStages * kMLd * sizeof(float);
-  if (rows >= 152 * 32 && t_bytes + wide_rows * 64 * x_row <= (size_t)kMWideSmem) {
+  if (rows >= 152 * 32 && t_bytes + most_rows * 64 * x_row <= (size_t)kMWideSmem) {
     const int64_t rpc = (rows + 151) / 152;
-    int rt = 8;
+    int rt = 8, wr = most_rows;
     int64_t best = INT64_MAX;
-    for (int r = 8; r >= 4; --r) {
-      const int64_t cost = (rpc + wide_rows * 8 * r - 1) / (wide_rows * 8 * r) * r;
-      if (cost < best) {
-        best = cost;
-        rt = r;
+    for (int w = most_rows; w >= 1; --w)
+      for (int r = 8; r >= 4; --r) {
+        // a tile's time goes with the rows of a thread, whatever the warps; of equal
+        // ones that with the fewest rows (its padding is copied too)
+        const int64_t cost = (rpc + w * 8 * r - 1) / (w * 8 * r) * r * 16 + w;
+        if (cost < best) {
+          best = cost;
+          rt = r;
+          wr = w;
+        }
       }
-    }
     auto k = rt == 8 ? k_gemm_wide<8> : rt == 7 ? k_gemm_wide<7> : rt == 6 ? k_gemm_wide<6>
              : rt == 5 ? k_gemm_wide<5> : k_gemm_wide<4>;
-    k<<<(unsigned)((rows + rpc - 1) / rpc), wide_rows * wcols * 32,
-        t_bytes + wide_rows * 8 * rt * x_row, s>>>(X, ldx, map, rows, rpc, T, kout, wide_rows, wcols,
-                                                   vec_x, vec_t, vec_y, Y, ldy);
+    k<<<(unsigned)((rows + rpc - 1) / rpc), wr * wcols * 32, t_bytes + wr * 8 * rt * x_row, s>>>(
+        X, ldx, map, rows, rpc, T, kout, wr, wcols, vec_x, vec_t, vec_y, Y, ldy);
     SFD_LAUNCH_CHECK();
     return;
   }
-  // else T through the stages: 64 rows per CTA (8 x 8 outputs per thread), 16 (2 x 8)
-  // where 64 would leave SMs without a CTA
-  const int rt = (rows + 63) / 64 < 2 * 152 ? 2 : 8, tile = 8 * rt;
+  // else T through the stages: 64 rows per CTA (8 x 8 outputs per thread), or 16 (2 x 8)
+  // below two CTAs an SM of 64. T, which every CTA loads, outweighs empty SMs from 193
+  // outputs on: 16 rows there only where 64 leave half of the SMs empty (256 x 256:
+  // 10,000 rows 67 us, 100 with 16 rows; 4,900 rows 39 and 53; 4,801 x 150 x 150 32 and 23)
+  const int64_t ctas64 = (rows + 63) / 64;
+  const int rt = ctas64 < (wcols >= 7 ? 76 : 2 * 152) ? 2 : 8, tile = 8 * rt;
   const size_t bytes = (size_t)kMStages * (tile * kMLd + kMK * wcols * 32) * sizeof(float);
   auto k = rt == 2 ? k_gemm_rows<2> : k_gemm_rows<8>;
   k<<<(unsigned)((rows + tile - 1) / tile), wcols * 32, bytes, s>>>(

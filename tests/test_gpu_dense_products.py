@@ -80,3 +80,17 @@ def test_dense_shrink_of_two_blocks(L, rows, ell):
     # compare the squares, at the 2e-5 n^1/2 / 4 ||M||^2 the eigensolver is held to
     tol = 2e-5 * max(1, np.sqrt(rows) / 4) * s[0] ** 2
     assert np.all(np.abs(got ** 2 - want ** 2) <= tol)
+
+
+# narrow outputs, whose CTAs take as many rows of warps as their rows need, and wide ones
+# on both sides of where 64 rows a CTA leave half of the SMs empty (4,800 rows)
+@pytest.mark.parametrize("n,kout,pad", [(50, 3, 0), (100, 20, 4), (200, 3, 1), (200, 20, 0),
+                                        (250, 33, 2), (255, 193, 1), (256, 224, 0), (193, 255, 0)])
+@pytest.mark.parametrize("rows", [2, 4799, 4801, 4863, 4865, 10000, 20011])
+def test_narrow_and_wide_products_are_exact_on_whole_numbers(L, n, kout, pad, rows):
+    X = block(rows, n, n + pad, 0, n + rows)
+    T = block(n, kout, kout, 0, kout)
+    Y = torch.full((rows + 1, kout), -7.0, device="cuda")
+    assert L.sfd_gemm_ts(rows, n, ptr(X), n + pad, ptr(T), kout, ptr(Y), kout, 0) == 0
+    assert torch.equal(Y[:rows].double(), X[:, :n].double() @ T.double())
+    assert torch.all(Y[rows:] == -7.0)
