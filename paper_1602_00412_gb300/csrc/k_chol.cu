@@ -21,10 +21,12 @@
 // diagonal block left 250 clocks per column on its shuffles.)
 //
 // Measured (GB300, back-to-back launches; column-at-a-time and 16-wide panel forms
-// with FP64 before): fp32 k = 50 / 100 / 200: 8 / 21 / 74 us (20 / 47 / 893), accurate
-// k = 50 / 100 / 200: 29 / 78 / 361 us (about 110 / 387 / 2408). The error of Rinv
-// against a double-precision factor of the same matrix is 1e-7 in fp32 and that of
-// the final rounding to fp32 (2e-8 to 3e-8) in the accurate form.
+// with FP64 before): fp32 k = 50 / 100 / 200: 8 / 20 / 71 us (20 / 47 / 893), accurate
+// k = 50 / 100 / 200: 30 / 76 / 345 us (about 110 / 387 / 2408). The error of Rinv
+// against a double-precision factor of the same matrix is, in the accurate form, that of
+// the final rounding to fp32 (2.1e-8 to 2.6e-8, as the FP64 factor's) up to condition
+// number 1e6 of G; in fp32 0.8e-7 to 1.4e-7 at condition 10 and 1e-3 to 1.8e-3 at 1e6
+// (0.8e-7 to 3.2e-7 and 1.5e-3 to 2.6e-3 before).
 //
 // The accurate passes (see chol_inv) hold every value as an unevaluated sum of
 // two floats (48 significant bits; sums and products by the error-free

@@ -77,8 +77,10 @@ __global__ void k_gauss_fill(float* __restrict__ out, int64_t rows, int cols, in
 // 4 (ng + g) + 3, so that neighbouring tiles' float4 loads use different banks with the
 // rows as they lie in memory. Rows arrive 16 at a time through a ring of cp.async
 // stages, as a straight copy where rows are contiguous (k_gram_tri). The multiply-adds
-// are packed two columns at a time (half the issue slots; each is rounded as fmaf) and
-// bound the kernel: 64 per thread and row against 4 shared float4 loads.
+// are packed two columns at a time (half the issue slots; each is rounded as fmaf), 64
+// per thread and row against 4 shared float4 loads. What bounds it is latency: with 64
+// accumulators a thread there are two warps per scheduler, and at 200,000 x 200 the FMA
+// pipe is 55 % busy, the shared-memory pipe 59 %.
 // Cold, with its reduction: 100,000 x 200 128 us (31 TFLOP/s, one triangle counted; 438
 // in 128 x 128 tiles, 168 with row by row copies), 20,000 x 100 23 us (49, 25), 2,000 x
 // 50 11 us (15 with row by row copies). Rows of any other alignment go row by row, their
@@ -369,10 +371,11 @@ __global__ void __launch_bounds__(32 * kRedGroups)
 // so its loads of X and T from shared memory are one wavefront each, 16 per 4 inner
 // columns against 256 multiply-adds per lane at RT = 8. X and T arrive 16 inner
 // columns at a time through a ring of cp.async stages (T from L2), T's rows split in
-// halves as the Gram's. Each output adds its products in column order. Bound by the
-// packed multiply-adds where there are rows enough: 50,000 x 200 x 200 takes 131 us
-// (31 TFLOP/s; 205 in 128 x 128 tiles, a fifth of their products padding), 20,000 x 100
-// x 100 27 us (46).
+// halves as the Gram's. Each output adds its products in column order. Where
+// there are rows enough 50,000 x 200 x 200 takes 131 us (31 TFLOP/s; 205 in 128 x 128
+// tiles, a fifth of their products padding), 20,000 x 100 x 100 27 us (46): the FMA pipe
+// is 58 % busy (200,000 x 200 x 200), because the warps come to it together after each
+// barrier and each step of four columns' loads.
 constexpr int kMK = 16;        // inner columns per stage
 constexpr int kMLd = kMK + 4;  // X stage leading dimension: 8 rows start in 8 bank quads
 constexpr int kMStages = 3;
