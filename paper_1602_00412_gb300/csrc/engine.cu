@@ -316,7 +316,7 @@ void Slot::build(int m, int64_t nnz, int64_t max_row) {
   csr.nseg = m;
   csr.nnz = nnz;
   csr.may_split = max_row < 0 || max_row > kSplit;
-  launch_check_entries(csr.idx, csr.val, nnz, (int)d, nullptr, fro2, ws.flags, stream);
+  launch_check_entries(csr.idx, csr.val, nnz, (int)d, csr.idx, nullptr, fro2, ws.flags, stream);
   build_work(csr, stream);
   build_csc(csr, csc, (int)d, sort, ws, stream);
 }

@@ -187,3 +187,30 @@ def test_scratch_given_back_without_a_sketch(sfd):
     assert torch.cuda.mem_get_info()[0] == free
     L.sfd_destroy(None)
     call()
+
+
+@pytest.mark.parametrize("bad", [-(2 ** 31), -70000, -7, 2500, 70000, 2 ** 31 - 1])
+def test_far_column_indices_are_refused(sfd, bad):
+    # the columns are sorted before the host has read the check's result: every index out
+    # of range must be harmless there, near or far, one or many
+    L = sfd.load()
+    for p in products():
+        i = p.dev[1]
+        for where in (slice(-1, None), slice(None)):
+            if not i.numel() or (bad >= 0 and bad < p.d):
+                continue
+            p.Y.fill_(-7.0)
+            ib = i.clone()
+            ib[where] = bad
+            assert p.call(L, idx=ib) == SFD_EINVAL
+            assert bool((p.Y == -7.0).all()) and bool((ib[where] == bad).all())
+        p.check(L)
+    m = d = 300
+    A = Product(list(np.random.default_rng(2).integers(1, 30, m)), d, 4, False, 9)
+    ib = A.dev[1].clone()
+    ib[::3] = bad
+    Bp = torch.full((20, d), -7.0, device="cuda")
+    with pytest.raises(sfd.SfdError) as e:
+        sfd.sfd_bssh_buffer(m, d, 20, A.dev[0], ib, A.dev[2], 1, 0, Bp)
+    assert e.value.code == SFD_EINVAL and bool((Bp == -7.0).all())
+    A.check(L)
