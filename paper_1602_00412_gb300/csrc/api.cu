@@ -387,7 +387,7 @@ int sfd_append_rows(sfd_ctx* ctx, int64_t nrows, const int64_t* indptr, const in
     }
     if (total > 0) {
       SFD_CUDA(cudaMemsetAsync(C.chk_flags, 0, sizeof(int), C.in_stream));
-      launch_check_entries(didx, dval, total, (int)C.d, nullptr, nullptr, C.chk_fro2, C.chk_flags,
+      launch_check_entries(didx, dval, total, (int)C.d, nullptr, C.chk_fro2, C.chk_flags,
                            C.in_stream);
       int bad = 0;
       SFD_CUDA(cudaMemcpyAsync(&bad, C.chk_flags, sizeof(int), cudaMemcpyDeviceToHost, C.in_stream));

@@ -316,16 +316,39 @@ void Slot::build(int m, int64_t nnz, int64_t max_row) {
   csr.nseg = m;
   csr.nnz = nnz;
   csr.may_split = max_row < 0 || max_row > kSplit;
-  launch_check_entries(csr.idx, csr.val, nnz, (int)d, csr.idx, nullptr, fro2, ws.flags, stream);
+  launch_check_entries(csr.idx, csr.val, nnz, (int)d, nullptr, fro2, ws.flags, stream);
   build_work(csr, stream);
   build_csc(csr, csc, (int)d, sort, ws, stream);
 }
+
+namespace {
+
+// The columns as sort keys, a copy of idx that replaces one outside [0, d) by 0: a stage
+// call queues the sort and the column pointer, which index by the key, before the host
+// has read whether the entries are good.
+__global__ void __launch_bounds__(256)
+    k_column_keys(const int* __restrict__ idx, int64_t n, int d, int* __restrict__ key) {
+  const int64_t first = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const int64_t i = first + t * 256;
+    if (i < n) {
+      const int c = idx[i];
+      key[i] = c >= 0 && c < d ? c : 0;
+    }
+  }
+}
+
+}  // namespace
 
 // by a stable radix sort of (col, row, val) by col
 void build_csc(const Csr& csr, Csr& csc, int d, const SortBuffers& t, const Workspace& ws,
                cudaStream_t s) {
   const int64_t nnz = csr.nnz;
-  SFD_CUDA(cudaMemcpyAsync(t.key, csr.idx, nnz * sizeof(int), cudaMemcpyDeviceToDevice, s));
+  if (nnz > 0) {
+    k_column_keys<<<(unsigned)((nnz + 1023) / 1024), 256, 0, s>>>(csr.idx, nnz, d, t.key);
+    SFD_LAUNCH_CHECK();
+  }
   SFD_CUDA(cudaMemcpyAsync(csc.val, csr.val, nnz * sizeof(float), cudaMemcpyDeviceToDevice, s));
   launch_row_ids(csr.ptr, csr.nseg, csc.idx, s);
   radix_sort_by_key(t.key, csc.idx, csc.val, t.key2, t.a, t.b, nnz, bits_for(d), ws.hist,

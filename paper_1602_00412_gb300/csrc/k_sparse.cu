@@ -46,10 +46,8 @@ __global__ void k_row_ids(const int* __restrict__ ptr, int nseg, int* __restrict
 // ------------------------------------------------------------ check + norms
 constexpr int kCheckBlocks = 1024;
 
-// repair: idx itself when it is the library's copy and kernels queued behind this one
-// index by it before the host reads the flag; an index outside [0, d) becomes 0 there
-__global__ void k_check_entries(const int* idx, const float* __restrict__ val, int64_t nnz, int d,
-                                int* repair, int* __restrict__ col_count,
+__global__ void k_check_entries(const int* __restrict__ idx, const float* __restrict__ val,
+                                int64_t nnz, int d, int* __restrict__ col_count,
                                 double* __restrict__ block_fro2, int* __restrict__ flags) {
   float acc = 0.f;
   int bad = 0;
@@ -59,7 +57,6 @@ __global__ void k_check_entries(const int* idx, const float* __restrict__ val, i
     float v = val[i];
     if (c < 0 || c >= d || !isfinite(v)) {
       bad = 1;
-      if (repair && (c < 0 || c >= d)) repair[i] = 0;
       continue;
     }
     if (col_count) atomicAdd(&col_count[c], 1);
@@ -586,11 +583,11 @@ void launch_row_ids(const int* ptr, int nseg, int* rows, cudaStream_t s) {
   SFD_LAUNCH_CHECK();
 }
 
-void launch_check_entries(const int* idx, const float* val, int64_t nnz, int d, int* repair,
-                          int* col_count, double* fro2_out, int* flags, cudaStream_t s) {
+void launch_check_entries(const int* idx, const float* val, int64_t nnz, int d, int* col_count,
+                          double* fro2_out, int* flags, cudaStream_t s) {
   // fro2_out[0] receives the total; fro2_out[1..kCheckBlocks] hold block partials
   int nb = (int)std::min<int64_t>(kCheckBlocks, std::max<int64_t>(1, (nnz + 1023) / 1024));
-  k_check_entries<<<nb, 256, 0, s>>>(idx, val, nnz, d, repair, col_count, fro2_out + 1, flags);
+  k_check_entries<<<nb, 256, 0, s>>>(idx, val, nnz, d, col_count, fro2_out + 1, flags);
   SFD_LAUNCH_CHECK();
   k_sum_doubles<<<1, 256, 0, s>>>(fro2_out + 1, nb, fro2_out);
   SFD_LAUNCH_CHECK();

@@ -144,7 +144,7 @@ int run_spmm(int64_t m, int64_t d, const int32_t* rowptr, const int32_t* colidx,
     csr.nseg = (int)m;
     csr.nnz = r.nnz;
     csr.may_split = r.max_row > kSplit;
-    launch_check_entries(csr.idx, csr.val, r.nnz, (int)d, csr.idx, nullptr, fro2, ws.flags, L->stream);
+    launch_check_entries(csr.idx, csr.val, r.nnz, (int)d, nullptr, fro2, ws.flags, L->stream);
     if (transposed) build_csc(csr, csc, (int)d, sort, ws, L->stream);
     else build_work(csr, L->stream);
     if (!entries_ok(*L.s, ws.flags)) return SFD_EINVAL;

@@ -125,10 +125,9 @@ struct Workspace {
 void launch_row_ids(const int* ptr, int nseg, int* rows, cudaStream_t s);
 // Validate a buffer slice: indices in [0,d), finite values; sum of squares
 // into fro2_out[0]; column counts (atomic) when col_count is not null. Sets
-// flags[0] on a bad index/value. repair (null or idx): bad indices become 0, so that
-// what is queued behind stays in bounds until the host has read the flag.
-void launch_check_entries(const int* idx, const float* val, int64_t nnz, int d, int* repair,
-                          int* col_count, double* fro2_out, int* flags, cudaStream_t s);
+// flags[0] on a bad index/value.
+void launch_check_entries(const int* idx, const float* val, int64_t nnz, int d, int* col_count,
+                          double* fro2_out, int* flags, cudaStream_t s);
 // ptr[c] = first position of column c in the column-sorted keys (ptr[d] = n).
 void colptr_from_sorted(const int* keys, int64_t n, int d, int* ptr, cudaStream_t s);
 // Exclusive scan of n ints (n >= 0) into out[0..n]; out[n] = total.
